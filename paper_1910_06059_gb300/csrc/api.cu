@@ -77,10 +77,11 @@ static void free_all(bo_sim* s) {
     destroy_graphs(s);
     cpr_free(s);
     dd_free(s);
+    free_sweeps64(s);
     learn_set_clear(s);
     void* ptrs[] = {s->d_dx, s->d_dy, s->d_dz, s->d_perm, s->d_poro, s->d_T, s->d_pv, s->d_depth,
                     s->d_p, s->d_sw, s->d_x, s->d_flag, s->d_bk, s->d_bkflag, s->d_A0,
-                    s->d_props, s->d_R, s->d_A, s->d_P, s->d_yt, s->d_qt, s->d_order, s->d_face, s->d_cellcon, s->d_wells,
+                    s->d_props, s->d_R, s->d_A, s->d_P, s->d_face, s->d_cellcon, s->d_wells,
                     s->d_con_cell, s->d_con_wi, s->d_wB, s->d_wC, s->d_b, s->d_xs, s->d_r,
                     s->d_rh, s->d_pk, s->d_v, s->d_s, s->d_t, s->d_ph, s->d_sh, s->d_part,
                     s->d_ks, s->d_ns, s->d_sweep_sync, s->d_P32, s->d_r32, s->d_y32,
@@ -393,9 +394,6 @@ bo_status bo_create_grid(int nx, int ny, int nz, const double* dx, const double*
             dalloc(&s->d_P, 63 * ilu_storage(s));
             // idle slots of the tile order are never written: zero factors
             BO_CUDA(cudaMemset(s->d_P, 0, sizeof(double) * 63 * ilu_storage(s)));
-            dalloc(&s->d_yt, 3 * ilu_storage(s));
-            dalloc(&s->d_qt, 3 * ilu_storage(s));
-            dalloc(&s->d_order, 2 * (size_t)tile_count(s));
             dalloc(&s->d_face, face_storage(s));
             dalloc(&s->d_sweep_sync, 4);
             for (double** v : {&s->d_b, &s->d_xs, &s->d_r, &s->d_rh, &s->d_pk, &s->d_v, &s->d_s,
@@ -967,9 +965,16 @@ bo_status bo_set_subdomains(bo_sim* s, int ysub, int zsub) {
         need(s->props_set, BO_ERR_STATE, "bo_set_subdomains: call bo_set_properties first");
         if (ysub == s->ysub && zsub == s->zsub) return;
         sync(s);
+        const int ysub0 = s->ysub, zsub0 = s->zsub;
         s->ysub = ysub;
         s->zsub = zsub;
-        update_sweep_order(s);
+        try {
+            setup_sweeps64(s);   // on failure the old plan stays
+        } catch (...) {
+            s->ysub = ysub0;
+            s->zsub = zsub0;
+            throw;
+        }
         s->factored = false;   // the factors of the other partition are stale
         reset_sweep_faces(s);
         build_graphs(s);
@@ -1141,6 +1146,8 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
         learn_setup_training(s);
         const auto t0 = std::chrono::steady_clock::now();
         const size_t N = 3 * (size_t)s->geo.n;
+        double first = 0.0, last = 0.0;
+        long long cnt = 0;
         // each kept system's Jacobian, ILU(0) data, features and scalings take
         // the place of the current ones while its residuals are trained on
         struct Swap {
@@ -1154,15 +1161,16 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
                 s->d_ml_featf = featf;
                 s->d_ml_cell = cell;
             }
-        } keep{s, s->d_A, s->d_P, s->d_ml_featf, s->d_ml_cell};
-        double first = 0.0, last = 0.0;
-        long long cnt = 0;
+        };
+        {
+        Swap keep{s, s->d_A, s->d_P, s->d_ml_featf, s->d_ml_cell};
         for (int ep = 0; ep < epochs; ++ep) {
             for (const LearnSystem& q : s->ml_set) {
                 s->d_A = q.A;
                 s->d_P = q.P;
                 s->d_ml_featf = q.featf;
                 s->d_ml_cell = q.cell;
+                enqueue_factor_lower(s, s->stream);   // the sweeps' copies of its factors
                 for (int j = 0; j < q.nr; ++j) {
                     const double L = learn_loss_grad(s, q.r + (size_t)j * N);
                     if (ep == 0) first += L;
@@ -1173,6 +1181,8 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
                 }
             }
         }
+        }
+        if (s->factored) enqueue_factor_lower(s, s->stream);
         sync(s);
         check_timeout(s);
         s->ml_train_ms +=
@@ -1357,7 +1367,7 @@ bo_status bo_set_sweep_ctas_per_sm(bo_sim* s, int k) {
         if (k == s->sweep_ctas_per_sm) return;
         sync(s);
         s->sweep_ctas_per_sm = k;
-        setup_sweeps64(s);   // residency check and tile lists for the new grid
+        reset_tickets(s);
         build_graphs(s);     // the captured launches carry the grid
     });
 }

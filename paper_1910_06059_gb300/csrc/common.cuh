@@ -120,6 +120,26 @@ struct LearnSystem {
     int nr = 0;
 };
 
+// FP64 sweeps (sweep64.cu): a tile of TSJ x TSK x-lines in one sweep direction
+// (lines counted in that direction), the tiles that read its results (-1:
+// none) and whether it reads the tiles before it; the plan of both directions
+// (0 forward, 1 backward) for the current block-Jacobi boxes.
+constexpr int TSJ = 4, TSK = 3;
+struct SweepTile {
+    int j0, k0, nextJ, nextK;
+    short nj, nk, depJ, depK;
+};
+struct SweepPlan {
+    int T = 0, NL = 0;
+    SweepTile* tiles[2] = {nullptr, nullptr};
+    unsigned* line[2] = {nullptr, nullptr};
+    double* S[2] = {nullptr, nullptr};      // scaled off-diagonal blocks, lane order
+    double* Q[2] = {nullptr, nullptr};      // right-hand sides
+    double* inbox = nullptr;
+    unsigned long long* ticket = nullptr;
+    double* Dn = nullptr;                   // D^-1 [9][n]
+};
+
 struct CprData;   // CPR preconditioner data (cpr.cu)
 struct DdData;    // K-subdomain solver data (dd.cu)
 
@@ -163,9 +183,7 @@ struct bo_sim {
     double* d_R = nullptr;       // 3n
     double* d_A = nullptr;       // 63n
     double* d_P = nullptr;       // 63 x tile-order ILU(0) data
-    double* d_yt = nullptr;      // forward-sweep result, tile order [slot][3][32]
-    double* d_qt = nullptr;      // forward-sweep right-hand side D^-1 r, tile order
-    int* d_order = nullptr;      // sweep tile lists: forward [T], backward [T]
+    bo::SweepPlan sweep;         // FP64 sweeps: tiles, factors, right-hand sides
     float* d_P32 = nullptr;      // FP32 factors in the FP32 sweep layout (mixed mode)
     float* d_r32 = nullptr;      // FP32 sweep input, tile order (mixed mode)
     float* d_y32 = nullptr;      // FP32 sweep work vector, tile order (mixed mode)
@@ -241,7 +259,7 @@ struct bo_sim {
     cudaGraphExec_t g_factor = nullptr;
     cudaGraphExec_t g_iter_timed = nullptr;
     int iters_per_graph = 4;
-    int sweep_ctas_per_sm = 2;   // persistent CTAs of the FP64 sweeps per SM (1 or 2)
+    int sweep_ctas_per_sm = 2;   // CTAs of the FP64 sweeps per SM (1 or 2)
     int ysub = 0;                // block-Jacobi slabs of ysub cell rows in y (0: no cut in y)
     int zsub = 0;                // and of zsub cell layers in z (0: no cut in z)
 
@@ -277,9 +295,10 @@ void launch_restore(bo_sim* s);
 void setup_sweeps(bo_sim* s);
 int sweep_timeout(bo_sim* s);
 size_t ilu_storage(const bo_sim* s);
-int tile_count(const bo_sim* s);                 // tiles of the wavefront schedule
-void update_sweep_order(bo_sim* s);              // sweep tile lists after a block-Jacobi change
-void setup_sweeps64(bo_sim* s);                  // FP64 sweep grid: residency check, tile lists
+void setup_sweeps64(bo_sim* s);                  // FP64 sweep plan for the current boxes
+void free_sweeps64(bo_sim* s);
+void reset_tickets(bo_sim* s);                   // after a change of the sweeps' grid
+void enqueue_factor_lower(bo_sim* s, cudaStream_t st);   // scaled lower blocks, sweep copies
 size_t face_storage(const bo_sim* s);
 void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad);
 void enqueue_fwd(bo_sim* s, cudaStream_t st, const double* r, double* y, const KrylovScalars* ks);

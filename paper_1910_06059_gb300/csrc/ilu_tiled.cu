@@ -25,9 +25,9 @@
 // the sweep finishes with zeros for the missing values.
 //
 // The factor data P is stored in tile order (pidx in tiles.cuh): a tile
-// level's 63 entries x 32 lanes are contiguous, so the sweeps move a level
-// with one bulk copy; b: 0 D^-1, 1..3 D^-1 A_{c,-x/-y/-z}, 4..6 D^-1
-// A_{c,+x/+y/+z}.  The sweeps themselves are in sweep64.cu.
+// level's 63 entries x 32 lanes are contiguous; b: 0 D^-1, 1..3 D^-1
+// A_{c,-x/-y/-z}, 4..6 D^-1 A_{c,+x/+y/+z}.  The FP64 sweeps (sweep64.cu) read
+// copies in their own order.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -231,9 +231,11 @@ k_factor_tiled(TileArgs a, const double* __restrict__ A, double* __restrict__ P,
 }
 
 // Scaled lower blocks D_c^-1 A_{c,-x/-y/-z} for every tile-order slot (one
-// thread per slot, full warps; zero for idle slots and missing neighbours).
+// thread per slot, full warps; zero for idle slots and missing neighbours),
+// and the copies the FP64 sweeps stream: both triangles in their lane order,
+// D^-1 in natural order.
 __global__ void __launch_bounds__(256)
-k_factor_lower(TileArgs a, const double* __restrict__ A, double* __restrict__ P) {
+k_factor_lower(TileArgs a, const double* __restrict__ A, double* __restrict__ P, SweepFactors f) {
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < a.NP;
          idx += (size_t)gridDim.x * blockDim.x) {
         const int lane = (int)(idx & 31);
@@ -243,9 +245,20 @@ k_factor_lower(TileArgs a, const double* __restrict__ A, double* __restrict__ P)
         const int j = J * TJ + jj, k = K * TK + kk, i = l - jj - kk;
         const bool act = j < a.g.ny && k < a.g.nz && i >= 0 && i < a.g.nx;
         const int c = act ? i + a.g.nx * (j + a.g.ny * k) : 0;
+        // this cell's places in the two sweeps' factors
+        double *sf = nullptr, *sb = nullptr;
+        if (act) {
+            const unsigned pf = f.fline[j + (size_t)a.g.ny * k], pb = f.bline[j + (size_t)a.g.ny * k];
+            const unsigned lf = pf / 36 + i, lb = pb / 36 - i, qf = pf % 36 / 3, qb = pb % 36 / 3;
+            sf = f.F + ((size_t)lf * TSJ + qf / TSK) * 96 + qf % TSK * 9;
+            sb = f.B + ((size_t)lb * TSJ + qb / TSK) * 96 + qb % TSK * 9;
+        }
         double Di[9], B[9], S[9];
 #pragma unroll
-        for (int e = 0; e < 9; ++e) Di[e] = act ? P[pidx(tl, e, lane)] : 0.0;
+        for (int e = 0; e < 9; ++e) {
+            Di[e] = act ? P[pidx(tl, e, lane)] : 0.0;
+            if (act) f.Dn[(size_t)e * a.g.n + c] = Di[e];
+        }
         const int lowb[3] = {NB_MX, NB_MY, NB_MZ};
         const bool keep[3] = {true, !ycut(a, j), !zcut(a, k)};
 #pragma unroll
@@ -255,7 +268,13 @@ k_factor_lower(TileArgs a, const double* __restrict__ A, double* __restrict__ P)
                 B[e] = act && keep[d] ? A[(size_t)(lowb[d] * 9 + e) * a.g.n + c] : 0.0;
             mm3t(Di, B, S);
 #pragma unroll
-            for (int e = 0; e < 9; ++e) P[pidx(tl, (1 + d) * 9 + e, lane)] = S[e];
+            for (int e = 0; e < 9; ++e) {
+                P[pidx(tl, (1 + d) * 9 + e, lane)] = S[e];
+                if (act) {
+                    sf[(e % 3) * 32 + (e / 3) * 3 + d] = S[e];
+                    sb[(e % 3) * 32 + (e / 3) * 3 + d] = P[pidx(tl, 36 + 9 * d + e, lane)];
+                }
+            }
         }
     }
 }
@@ -292,10 +311,6 @@ TileArgs tile_args(const bo_sim* s) {
     a.ysub = s->ysub;
     a.zsub = s->zsub;
     return a;
-}
-
-int tile_count(const bo_sim* s) {
-    return ((s->geo.ny + TJ - 1) / TJ) * ((s->geo.nz + TK - 1) / TK);
 }
 
 size_t ilu_storage(const bo_sim* s) {
@@ -352,31 +367,31 @@ void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad) {
     launch_coop(st, tile_grid(s), 32 * TILE_WARPS, k_factor_tiled, a, (const double*)s->d_A,
                 s->d_P, faceJ9(s), faceK9(s), bad);
     count_launch(s, st);
-    k_factor_lower<<<152 * 8, 256, 0, st>>>(a, (const double*)s->d_A, s->d_P);
-    count_launch(s, st);
+    enqueue_factor_lower(s, st);
     if (s->mixed) convert_factors32(s, st);
 }
 
-static void refill_faces3(bo_sim* s, cudaStream_t st) {
-    TileArgs a = tile_args(s);
-    k_fill_sentinel<<<304, 256, 0, st>>>(faceJ3(s), (size_t)a.T * s->geo.nx * (TK + TJ) * 3);
+void enqueue_factor_lower(bo_sim* s, cudaStream_t st) {
+    k_factor_lower<<<152 * 8, 256, 0, st>>>(tile_args(s), (const double*)s->d_A, s->d_P,
+                                            sweep_factors(s));
     count_launch(s, st);
+    BO_LAUNCH_CHECK("k_factor_lower");
 }
 
-// Sentinels of the current precision in the 3-value face buffers (after a
-// precision switch or an abandoned sweep).
+// Sentinels of the current precision's sweeps (after a precision switch or an
+// abandoned sweep).
 void reset_sweep_faces(bo_sim* s) { fill_sweep_faces(s, s->mixed); }
 
 void fill_sweep_faces(bo_sim* s, bool fp32) {
     if (fp32)
         reset_faces32(s, s->stream);
     else
-        refill_faces3(s, s->stream);
+        reset_inbox(s, s->stream);
     BO_LAUNCH_CHECK("fill_sweep_faces");
 }
 
-// The forward sweep leaves y in a tile-order work vector (FP64: d_yt; mixed
-// mode: the FP32 one) and the backward sweep writes z in natural order; the
+// The forward sweep leaves y in the backward sweep's order (a work vector of its
+// own in either precision) and the backward sweep writes z in natural order; the
 // two always run as a pair (y is not needed in natural order).
 void enqueue_fwd(bo_sim* s, cudaStream_t st, const double* r, double* y, const KrylovScalars* ks) {
     (void)y;

@@ -5,70 +5,78 @@
 //   forward  y_c = D_c^-1 r_c - sum_lower (D_c^-1 A_ck) y_k
 //   backward z_c = y_c       - sum_upper (D_c^-1 A_cj) z_j
 //
-// Wavefront over tiles of TJ x TK x-lines, as in the factorisation: at tile
-// level l, lane (jj, kk) of a tile handles cell i = l - jj - kk, so the three
-// lower (upper) neighbours of its cell were handled one level earlier (later)
-// by the lane itself, by lane jj -+ 1 and by lane kk -+ 1, or by the
-// neighbouring tile for the lanes on the tile's faces.
+// The backward sweep is the forward sweep of the mirrored grid (i, j, k ->
+// nx-1-i, ny-1-j, nz-1-k), so one kernel does both: cell (i, j, k) takes its
+// three neighbours i-1, j-1, k-1 of its own direction.
 //
-// GB300 design.  An FP64 warp instruction holds its SM sub-partition for
-// about 64 cycles however many lanes are active, so a tile level costs what
-// its FP64 instructions cost; everything else is kept off that path:
-//   * q = D^-1 r is formed before the wavefront by a fully parallel kernel,
-//     in tile order; one CTA of four warps per tile; warps 0-2 compute rows
-//     0-2 of the level (three block products, two FMA chains), each on its
-//     own sub-partition; warp 3 (the helper) fetches the face values of the
-//     neighbouring tiles and keeps the stage ring full;
-//   * the factor rows of a tile level are one contiguous chunk in HBM
-//     (ILU data in tile order, 63 entries x 32 lanes per level) and reach
-//     shared memory by cp.async.bulk copies (the level's three scaled
-//     blocks and its 3-vector q or y) into a ring of S64 stages, each
-//     completed on its own mbarrier, S64 - 1 levels ahead of the arithmetic;
-//   * the level's results are exchanged through a zero-padded plane in
-//     shared memory whose border row and column hold the neighbouring tiles'
-//     face values (written by the helper), so every lane reads its three
-//     neighbours with the same three loads: no selects, no shuffles;
-//   * the CTAs are persistent: 2 per SM, each taking its tiles from a list in
-//     topological order (sorted by the level at which a tile can start);
-//     the ring runs on across a CTA's tiles.  A tile waits only for tiles
-//     earlier in the list, every CTA is resident (cooperative launch), so
-//     every wait ends;
-//   * face values pass through write-once slots holding a NaN sentinel; the
-//     helper polls (bounded) until a value appears and puts the sentinel back,
-//     so no refill kernel runs between sweeps.
-// Idle slots of the tile order (ragged tiles, i outside the line) hold zero
-// factors; inactive lanes produce zero, so the padding needs no predicates
-// in the arithmetic.  The forward result y stays in tile order (the
-// backward sweep's bulk copies read it); the backward result z is written in
-// natural order.
+// What bounds it.  The recurrence runs over nx + ny + nz - 2 wavefront levels
+// (363 on the 60x220x85 model).  An FP64 warp instruction takes 64 cycles, in
+// throughput of its sub-partition and in latency, and an SM issues one in 19
+// cycles, so a level costs its longest chain of FP64 operations, plus what is
+// lost between levels.  Bytes do not bind: the 350 MB a sweep moves on that
+// model take 51 us.
+//   * A cell's row is u + (v + w): three chains of three products, one per
+//     neighbour.  Each chain has its own lane (9 lanes a cell, 3 cells a
+//     warp), so a level is 3 dependent products and 2 additions, 5 x 77 cycles
+//     with four warps; three chains in one lane would be 11 operations.
+//   * A CTA has four such warps (one per sub-partition) and a tile of 4 x 3
+//     x-lines (TSJ x TSK); at tile level l, line (jj, kk) handles cell i = l - jj
+//     - kk.  Results pass through a small plane in shared memory, one barrier a
+//     level; a level of a tile on its own takes 619 cycles, 314 ns.
+//   * The factors are stored lane by lane, a level's 3 KB in one piece: a copy
+//     warp brings them and the right-hand side into a ring in shared memory with
+//     two bulk copies a level, RING levels ahead (cp.async by the compute warps
+//     instead: 343 ns a level; plain loads six levels ahead: 400 ns).
+//   * Values of the neighbouring tiles come through write-once slots in global
+//     memory that hold a NaN sentinel until written.  Four face warps poll them,
+//     each every fourth level, write them to a ring in shared memory and arrive
+//     at the barrier that opens their level, so a round trip to L2 (0.47 us one
+//     way between two SMs) is paid once per tile crossing, 0.73 us in all, and
+//     not once per level.
+//   * CTAs take tiles from a ticket counter in topological order (sorted by the
+//     level at which a tile can start).  A tile waits only for tiles with smaller
+//     tickets, which CTAs already running hold, so every wait ends whatever else
+//     shares the GPU and no launch has to be resident as a whole.
+// Measured, a sweep: 60x220x85 265 us (405 before, with one warp per row of an
+// 8 x 4 tile and a handoff per level), 33x27x9 31 us (52.6 before).
+// Waits are bounded; one that runs out sets the error flag and the sweep ends
+// with zeros for the missing values.
 #include <algorithm>
+#include <tuple>
 #include <vector>
 
 #include "tiles.cuh"
 
 namespace bo {
 
-constexpr int S64 = 8;                          // stages of the ring
-constexpr int SW_THREADS = 128;                 // 3 row warps + the helper warp
-constexpr int HELPER = 3;                       // warp index of the helper
-constexpr int BLK_ENT = 27;                     // 3 scaled off-diagonal blocks
-constexpr int STAGE = (BLK_ENT + 3) * 32;       // doubles per stage: blocks + a 3-vector
-constexpr int HJ = TJ + 1, HK = TK + 1;         // padded exchange plane
-constexpr int YPL = HK * HJ;                    // one component of the plane
-constexpr int YBUF = 3 * YPL;                   // one level of the plane
-constexpr long long MBAR_LIMIT64 = 1LL << 22;   // bounded mbarrier waits
+constexpr int FACE_WARPS = 4;             // each opens every fourth level
+constexpr int SWEEP_THREADS = 32 * (TSJ + FACE_WARPS + 1);   // and the copy warp
+constexpr int WAIT_LIMIT = 1 << 26;       // polls of a level counter (several seconds)
+constexpr int LINES = TSJ * TSK;          // x-lines of a tile
+constexpr int RING = 8;                   // levels of the rings (power of two)
+constexpr int STAGE = 96 * TSJ + 3 * TSJ * TSK;   // doubles of a level: factors, right-hand side
+constexpr int SLOT = 3 * LINES;           // doubles of one level in shared memory
+constexpr int FACE_LANES = 3 * (TSK + TSJ);   // face values of one level: j-face, k-face
+static_assert(TSJ == 4 && TSK == 3, "one warp per j-line of the tile, three lines a warp");
+static_assert(TSJ + TSK <= LINES && FACE_LANES <= FACE_W, "a level's face values fit a slot");
 
-// ---------------------------------------------------------------------------
-// mbarrier and bulk-copy primitives (PTX)
-// ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned sa(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
-__device__ __forceinline__ void mb_init(unsigned long long* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sa(bar)), "r"(count) : "memory");
+// Level counters in shared memory.  Plain volatile accesses: a warp's shared
+// memory accesses are performed in order, and a release would also wait for the
+// warp's global stores under way (several hundred cycles a level).
+__device__ __forceinline__ int ld_level(const int* p) {
+    int v;
+    asm volatile("ld.volatile.shared.b32 %0, [%1];" : "=r"(v) : "r"(sa(p)) : "memory");
+    return v;
 }
-__device__ __forceinline__ void mb_fence_init() {
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+__device__ __forceinline__ void st_level(int* p, int v) {
+    asm volatile("st.volatile.shared.b32 [%0], %1;" ::"r"(sa(p)), "r"(v) : "memory");
+}
+// mbarriers of the stages and the copies that complete them
+__device__ __forceinline__ void mb_init(unsigned long long* bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sa(bar)) : "memory");
 }
 __device__ __forceinline__ void mb_expect(unsigned long long* bar, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(bar)), "r"(bytes)
@@ -84,27 +92,7 @@ __device__ __forceinline__ bool mb_try(unsigned long long* bar, unsigned parity)
         : "memory");
     return ok != 0;
 }
-// Bounded wait for a stage; gives up at once when another wait of the sweep
-// has already given up (the error flag is set), so a failed sweep ends fast.
-__device__ __forceinline__ bool mb_test(unsigned long long* bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(sa(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void mb_wait(unsigned long long* bar, unsigned parity, int* err) {
-    if (mb_test(bar, parity)) return;   // the usual case: the copy landed levels ago
-    for (long long q = 0; q < MBAR_LIMIT64; ++q) {
-        if (mb_try(bar, parity)) return;
-        if ((q & 1023) == 1023 && ld_relaxed_i(err) != 0) return;
-    }
-    atomicExch(err, 1);
-}
-// global -> shared bulk copy (16-byte aligned addresses, size a multiple of 16)
+// global -> shared (16-byte aligned addresses, a multiple of 16 bytes)
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes,
                                          unsigned long long* bar) {
     asm volatile(
@@ -113,515 +101,419 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
         "l"(src), "r"(bytes), "r"(sa(bar))
         : "memory");
 }
-
-struct SweepArgs {
-    TileArgs a;
-    const int* order;   // tiles in topological order of the sweep's direction
-    int G;              // CTAs of the launch
-};
-
-// Geometry of one lane of tile t.
-struct LaneGeo {
-    int t, J, K, j, k, l0, cbase;   // cell at level l: cbase + l (when active)
-    bool valid;
-};
-__device__ __forceinline__ LaneGeo lane_geo(const TileArgs& a, int t, int lane) {
-    LaneGeo G;
-    G.t = t;
-    G.J = t % a.NJ;
-    G.K = t / a.NJ;
-    const int jj = lane % TJ, kk = lane / TJ;
-    G.j = G.J * TJ + jj;
-    G.k = G.K * TK + kk;
-    G.l0 = jj + kk;
-    G.valid = G.j < a.g.ny && G.k < a.g.nz;
-    G.cbase = a.g.nx * (G.j + a.g.ny * G.k) - G.l0;
-    return G;
+// Opening of a level, on one of RING barriers in turn: its face warp arrives
+// (possibly several levels early), the compute warps wait.  The forms that
+// count threads: a warp that has come apart at a branch must not arrive twice.
+constexpr int OPEN = 32 * (TSJ + 1);
+__device__ __forceinline__ void level_sync(int place) {
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(1 + place), "n"(OPEN) : "memory");
 }
-__device__ __forceinline__ bool lane_active(const TileArgs& a, const LaneGeo& G, int l) {
-    const int i = l - G.l0;
-    return G.valid && i >= 0 && i < a.g.nx;
+__device__ __forceinline__ void level_arrive(int place) {
+    asm volatile("barrier.cta.arrive %0, %1;" ::"r"(1 + place), "n"(OPEN) : "memory");
 }
-
-// Poll a face slot (bounded) until none of its three values is the sentinel,
-// then put the sentinel back.  v holds the prefetched values on entry.
-__device__ __forceinline__ void take_slot(double* slot, double v[3], int* err) {
-    if (is_sentinel(v[0]) || is_sentinel(v[1]) || is_sentinel(v[2])) {
-        unsigned ns = 32;
-        for (long long q = 0;; ++q) {
-            v[0] = ld_relaxed(slot);
-            v[1] = ld_relaxed(slot + 1);
-            v[2] = ld_relaxed(slot + 2);
-            if (!is_sentinel(v[0]) && !is_sentinel(v[1]) && !is_sentinel(v[2])) break;
-            if (q >= POLL_LIMIT * 4 || ((q & 255) == 255 && ld_relaxed_i(err) != 0)) {
-                atomicExch(err, 1);
-                v[0] = v[1] = v[2] = 0.0;
-                return;
-            }
-            if (q >= 32) {
-                __nanosleep(ns);
-                ns = ns < 256u ? 2u * ns : 256u;
-            }
-        }
-    }
-    const double sent = __longlong_as_double((long long)SENTINEL_BITS);
-    st_relaxed(slot, sent);
-    st_relaxed(slot + 1, sent);
-    st_relaxed(slot + 2, sent);
-}
-
-// A helper lane's face slot for one tile: at level l the slot is
-// base + (l - off) stride, to be read when need and 0 <= l - off < nx; hp is
-// the slot's place in the padded exchange plane (-1: this lane has no face).
-struct FaceLane {
-    double* base;
-    int off, stride, hp;
-    bool need;
-};
-// Forward: lanes 0..TK-1 take the j-face of row kk = lane from tile J - 1,
-// lanes TK..TK+TJ-1 the k-face of column jj = lane - TK from tile K - 1.
-__device__ __forceinline__ FaceLane face_lane_fwd(const TileArgs& a, const LaneGeo& G, int lane,
-                                                  double* fJ, double* fK) {
-    FaceLane f{nullptr, 0, 0, -1, false};
-    if (lane < TK) {
-        const int kk = lane;
-        f.off = kk;
-        f.stride = TK * 3;
-        f.hp = (kk + 1) * HJ;
-        f.need = G.J > 0 && !ycut(a, G.J * TJ) && G.K * TK + kk < a.g.nz;
-        if (f.need) f.base = fJ + jslot(a, G.t - 1, 0, kk, 3);
-    } else if (lane < TK + TJ) {
-        const int jj = lane - TK;
-        f.off = jj;
-        f.stride = TJ * 3;
-        f.hp = jj + 1;
-        f.need = G.K > 0 && !zcut(a, G.K * TK) && G.J * TJ + jj < a.g.ny;
-        if (f.need) f.base = fK + kslot(a, G.t - a.NJ, 0, jj, 3);
-    }
-    return f;
-}
-// Backward: the upper neighbours of lane (TJ - 1, kk) in tile J + 1 and of
-// lane (jj, TK - 1) in tile K + 1.
-__device__ __forceinline__ FaceLane face_lane_bwd(const TileArgs& a, const LaneGeo& G, int lane,
-                                                  double* fJ, double* fK) {
-    FaceLane f{nullptr, 0, 0, -1, false};
-    if (lane < TK) {
-        const int kk = lane;
-        f.off = TJ - 1 + kk;
-        f.stride = TK * 3;
-        f.hp = kk * HJ + TJ;
-        f.need = G.J + 1 < a.NJ && !ycut(a, (G.J + 1) * TJ) && G.K * TK + kk < a.g.nz;
-        if (f.need) f.base = fJ + jslot(a, G.t + 1, 0, kk, 3);
-    } else if (lane < TK + TJ) {
-        const int jj = lane - TK;
-        f.off = jj + TK - 1;
-        f.stride = TJ * 3;
-        f.hp = TK * HJ + jj;
-        f.need = G.K + 1 < a.NK && !zcut(a, (G.K + 1) * TK) && G.J * TJ + jj < a.g.ny;
-        if (f.need) f.base = fK + kslot(a, G.t + a.NJ, 0, jj, 3);
-    }
-    return f;
-}
-__device__ __forceinline__ double* face_at(const FaceLane& f, int l, int nx) {
-    const int i = l - f.off;
-    return (f.need && i >= 0 && i < nx) ? f.base + (size_t)i * f.stride : nullptr;
-}
-
-// The helper warp's view of one stage: which tile and level it belongs to.
-struct StageCursor {
-    int m, l;   // m-th tile of this CTA, level (forward) or step (backward)
-};
-__device__ __forceinline__ void advance(StageCursor& c, int NL) {
-    if (++c.l == NL) {
-        c.l = 0;
-        ++c.m;
-    }
-}
-
-constexpr int MAX_CTA_TILES = 64;   // tiles of one CTA (checked on the host)
 
 // ---------------------------------------------------------------------------
-// q = D^-1 r in tile order, Qt[slot][3][32] (zero for idle slots): the
-// forward sweep's right-hand side, formed by all SMs before the wavefront.
-// Threads follow the tile order (a warp is one tile level), so the factor
-// reads and the writes are coalesced; neighbouring warps are neighbouring
-// levels of one tile and reuse each other's sectors of r.
+// q = D^-1 r in the forward sweep's order: its right-hand side, formed by all
+// SMs before the wavefront (9 products a cell, bound by bytes: 72 + 24 in, 24
+// out).  Idle slots keep the zeros they were allocated with.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-k_q_tiles(TileArgs a, const double* __restrict__ P, const double* __restrict__ r,
-          double* __restrict__ Qt, const KrylovScalars* __restrict__ ks) {
+k_sweep_rhs(int n, int nx, const unsigned* __restrict__ lb, const double* __restrict__ Dn,
+            const double* __restrict__ r, double* __restrict__ Q,
+            const KrylovScalars* __restrict__ ks) {
     if (ks_skip_t(ks)) return;
-    const int n = a.g.n;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < a.NP;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int lane = (int)(idx & 31);
-        const size_t slot = idx >> 5;
-        const int t = (int)(slot / a.NL), l = (int)(slot % a.NL);
-        const LaneGeo G = lane_geo(a, t, lane);
-        double rv[3] = {0.0, 0.0, 0.0};
-        if (lane_active(a, G, l)) {
-            const int c = G.cbase + l;
-#pragma unroll
-            for (int e = 0; e < 3; ++e) rv[e] = r[(size_t)e * n + c];
-        }
-        const double* D = P + slot * (NPE * 32) + lane;
-        double* q = Qt + slot * 96 + lane;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
+        const int jk = c / nx, i = c - jk * nx;
+        const double r0 = r[c], r1 = r[(size_t)n + c], r2 = r[2 * (size_t)n + c];
+        double* q = Q + lb[jk] + (size_t)i * SLOT;
 #pragma unroll
         for (int row = 0; row < 3; ++row) {
-            double v = D[(3 * row) * 32] * rv[0];
-            v = fma(D[(3 * row + 1) * 32], rv[1], v);
-            v = fma(D[(3 * row + 2) * 32], rv[2], v);
-            q[row * 32] = v;
+            double v = Dn[(size_t)(3 * row) * n + c] * r0;
+            v = fma(Dn[(size_t)(3 * row + 1) * n + c], r1, v);
+            v = fma(Dn[(size_t)(3 * row + 2) * n + c], r2, v);
+            q[row] = v;
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// a8 forward sweep: Yt = (L_A + D)^-1 r, from Qt = D^-1 r; Yt in tile order.
-// Row warp rw of a level: acc = q[rw] - L_x[rw][:] y_{i-1} - L_y[rw][:] y_{j-1}
-// - L_z[rw][:] y_{k-1} (ten FP64 operations in two chains).  A stage is the
-// level's three scaled lower blocks and q; the helper stages the face values
-// and issues the bulk copies.
+// a8: one sweep.  Compute warp w owns the lines jj = w, lane 9 kk + 3 row + d
+// the chain of row `row` towards neighbour d (0: i-1, 1: j-1, 2: k-1).
+// FWD writes y in the backward sweep's order, else z in natural order.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(SW_THREADS, 2)
-k_fwd64(SweepArgs A, const double* __restrict__ P, const double* __restrict__ Qt,
-        double* __restrict__ Yt, double* __restrict__ fJ, double* __restrict__ fK,
+template <bool FWD>
+__global__ void __launch_bounds__(SWEEP_THREADS, 2)
+k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
+        const unsigned* __restrict__ lbout, double* __restrict__ out,
         const KrylovScalars* __restrict__ ks) {
     if (ks_skip_t(ks)) return;
-    extern __shared__ __align__(128) double smem[];
-    double* ring = smem;                                   // [S64][STAGE]
-    double* ysh = ring + S64 * STAGE;                      // [2][3][HK][HJ]
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(ysh + 2 * YBUF);
-    int* tiles = reinterpret_cast<int*>(bar + S64);        // [MAX_CTA_TILES]
-    const TileArgs& a = A.a;
+    // PLANE: results of the last two levels [comp][kk TSJ + jj]; HALO: face
+    // values of RING levels [comp][kk | TSK + jj]; ZERO: no neighbour
+    constexpr int PLANE = 0, HALO = 2 * SLOT, ZERO = HALO + RING * SLOT;
+    __shared__ double ex[ZERO + SLOT];
+    __shared__ __align__(16) double ring[RING][STAGE];   // a level's factors and right-hand side
+    __shared__ unsigned long long bar[RING];
+    __shared__ unsigned s_rank;
+    __shared__ int s_done, s_begun;           // levels begun by the compute warps; level 0 is in
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int jj = lane % TJ, kk = lane / TJ;
-    const int NL = a.NL;
-    const int ntiles = blockIdx.x < a.T ? (a.T - 1 - blockIdx.x) / A.G + 1 : 0;
-    const long long total = (long long)ntiles * NL;
-    for (int q = threadIdx.x; q < ntiles; q += SW_THREADS) tiles[q] = A.order[blockIdx.x + q * A.G];
-    for (int q = threadIdx.x; q < 2 * YBUF; q += SW_THREADS) ysh[q] = 0.0;
-    __syncthreads();
-    // issue cursor (helper lane 0): stage (tile m, level l) copies slot t NL + l
-    StageCursor ic{0, 0};
-    size_t islot = (size_t)tiles[0] * NL;
-    long long issued = 0;
-    auto issue = [&]() {
-        const int st = (int)(issued % S64);
-        mb_expect(&bar[st], STAGE * 8);
-        double* dst = ring + (size_t)st * STAGE;
-        bulk_g2s(dst, P + islot * (NPE * 32) + 9 * 32, BLK_ENT * 32 * 8, &bar[st]);
-        bulk_g2s(dst + BLK_ENT * 32, Qt + islot * 96, 96 * 8, &bar[st]);
-        ++issued;
-        advance(ic, NL);
-        if (ic.l == 0) {
-            if (ic.m < ntiles) islot = (size_t)tiles[ic.m] * NL;
-        } else {
-            ++islot;
-        }
-    };
-    if (threadIdx.x == HELPER * 32) {
-        for (int d = 0; d < S64; ++d) mb_init(&bar[d], 1);
-        mb_fence_init();
-        while (issued < S64 - 1 && issued < total) issue();
-    }
-    __syncthreads();
-    if (total == 0) return;
+    const int NL = a.NL, nx = a.g.nx, n = a.g.n;
 
-    if (warp == HELPER) {
-        // ---- helper: face values and the ring -------------------------------
-        StageCursor nx{0, 0};   // the stage being prepared
-        LaneGeo G = lane_geo(a, tiles[0], lane);
-        FaceLane F = face_lane_fwd(a, G, lane, fJ, fK);
-        double fv[3] = {0.0, 0.0, 0.0};
-        auto load_faces = [&](int l) {
-            const double* sl = face_at(F, l, a.g.nx);
-#pragma unroll
-            for (int e = 0; e < 3; ++e) fv[e] = sl ? ld_relaxed(sl + e) : 0.0;
-        };
-        auto prepare = [&](long long g) {   // face values of stage g into the plane it reads
-            double* sl = face_at(F, nx.l, a.g.nx);
-            if (sl) take_slot(sl, fv, a.err);
-            if (F.hp >= 0) {
-                double* yb = ysh + (((int)(g & 1)) ^ 1) * YBUF + F.hp;
-                yb[0] = fv[0];
-                yb[YPL] = fv[1];
-                yb[2 * YPL] = fv[2];
-            }
-            advance(nx, NL);
-            if (g + 1 < total) {
-                if (nx.l == 0) {
-                    G = lane_geo(a, tiles[nx.m], lane);
-                    F = face_lane_fwd(a, G, lane, fJ, fK);
-                }
-                load_faces(nx.l);
-            }
-        };
-        // A tile's first stage is prepared only after the previous tile has
-        // finished (the barrier before it): the helper then waits only for
-        // tiles earlier in the list than the one the CTA is working on.
-        load_faces(0);
-        long long g = 0;
-        for (int m = 0; m < ntiles; ++m) {
-            prepare(g);
-            __syncthreads();
-            for (int l = 0; l < NL; ++l, ++g) {
-                if (lane == 0 && issued < total) issue();
-                if (l + 1 < NL) prepare(g + 1);
-                __syncthreads();
-            }
-        }
-        return;
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < RING; ++q) mb_init(&bar[q]);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-
-    // ---- row warps ---------------------------------------------------------
-    const int rw = warp;
-    const int op = (kk + 1) * HJ + jj + 1;   // this lane in the padded plane
-    long long g = 0;
-    for (int m = 0; m < ntiles; ++m) {
-        __syncthreads();   // the helper has prepared the tile's first stage
-        const LaneGeo G = lane_geo(a, tiles[m], lane);
-        const bool feedJ = G.valid && jj == TJ - 1 && G.J + 1 < a.NJ && !ycut(a, (G.J + 1) * TJ);
-        const bool feedK = G.valid && kk == TK - 1 && G.K + 1 < a.NK && !zcut(a, (G.K + 1) * TK);
-        double* yout = Yt + ((size_t)G.t * NL * 3 + rw) * 32 + lane;
-        double* fjo = fJ + jslot(a, G.t, 0, kk, 3) + rw - (size_t)G.l0 * TK * 3;
-        double* fko = fK + kslot(a, G.t, 0, jj, 3) + rw - (size_t)G.l0 * TJ * 3;
-        for (int l = 0; l < NL; ++l, ++g) {
-            const int st = (int)(g % S64);
-            mb_wait(&bar[st], (unsigned)((g / S64) & 1), a.err);
-            const double* L = ring + (size_t)st * STAGE + 3 * rw * 32 + lane;   // row rw of D^-1 A_-x
-            const double* yb = ysh + (((int)(g & 1)) ^ 1) * YBUF + op;
-            // three independent chains (q and the -x block, the -y block, the -z
-            // block) of three dependent FP64 operations each, then two adds
-            double u = ring[(size_t)st * STAGE + (BLK_ENT + rw) * 32 + lane];
-            double v = -L[9 * 32] * yb[-1];
-            double w = -L[18 * 32] * yb[-HJ];
-#pragma unroll
-            for (int s2 = 0; s2 < 3; ++s2) u = fma(-L[s2 * 32], yb[s2 * YPL], u);          // -x
-#pragma unroll
-            for (int s2 = 1; s2 < 3; ++s2) v = fma(-L[(9 + s2) * 32], yb[s2 * YPL - 1], v);   // -y
-#pragma unroll
-            for (int s2 = 1; s2 < 3; ++s2) w = fma(-L[(18 + s2) * 32], yb[s2 * YPL - HJ], w); // -z
-            const bool act = lane_active(a, G, l);
-            const double acc = act ? u + (v + w) : 0.0;
-            ysh[(int)(g & 1) * YBUF + rw * YPL + op] = acc;
-            yout[(size_t)l * 96] = acc;
-            if (act && feedJ) st_relaxed(fjo + (size_t)l * TK * 3, acc);
-            if (act && feedK) st_relaxed(fko + (size_t)l * TJ * 3, acc);
-            __syncthreads();
+    for (int turn = 0;; ++turn) {   // tiles this CTA has done
+        if (threadIdx.x == 0) {
+            s_rank = (unsigned)(atomicAdd(a.ticket, 1ull) % (unsigned long long)(a.T + gridDim.x));
+            s_done = s_begun = 0;
         }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// a8 backward sweep: z = (D + U_A)^-1 D y, y from Yt (tile order), z natural.
-// Levels run downward; the tile list is the forward list reversed.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(SW_THREADS, 2)
-k_bwd64(SweepArgs A, const double* __restrict__ P, const double* __restrict__ Yt,
-        double* __restrict__ z, double* __restrict__ fJ, double* __restrict__ fK,
-        const KrylovScalars* __restrict__ ks) {
-    if (ks_skip_t(ks)) return;
-    extern __shared__ __align__(128) double smem[];
-    double* ring = smem;                                   // [S64][STAGE]
-    double* ysh = ring + S64 * STAGE;                      // [2][3][HK][HJ]
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(ysh + 2 * YBUF);
-    int* tiles = reinterpret_cast<int*>(bar + S64);        // [MAX_CTA_TILES]
-    const TileArgs& a = A.a;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int jj = lane % TJ, kk = lane / TJ;
-    const int NL = a.NL, n = a.g.n;
-    const int ntiles = blockIdx.x < a.T ? (a.T - 1 - blockIdx.x) / A.G + 1 : 0;
-    const long long total = (long long)ntiles * NL;
-    for (int q = threadIdx.x; q < ntiles; q += SW_THREADS) tiles[q] = A.order[blockIdx.x + q * A.G];
-    for (int q = threadIdx.x; q < 2 * YBUF; q += SW_THREADS) ysh[q] = 0.0;
-    __syncthreads();
-    // issue cursor: stage (tile m, step l) copies slot t NL + NL - 1 - l
-    StageCursor ic{0, 0};
-    size_t islot = (size_t)tiles[0] * NL + NL - 1;
-    long long issued = 0;
-    auto issue = [&]() {
-        const int st = (int)(issued % S64);
-        mb_expect(&bar[st], STAGE * 8);
-        double* dst = ring + (size_t)st * STAGE;
-        bulk_g2s(dst, P + islot * (NPE * 32) + 36 * 32, BLK_ENT * 32 * 8, &bar[st]);
-        bulk_g2s(dst + BLK_ENT * 32, Yt + islot * 96, 96 * 8, &bar[st]);
-        ++issued;
-        advance(ic, NL);
-        if (ic.l == 0) {
-            if (ic.m < ntiles) islot = (size_t)tiles[ic.m] * NL + NL - 1;
-        } else {
-            --islot;
-        }
-    };
-    if (threadIdx.x == HELPER * 32) {
-        for (int d = 0; d < S64; ++d) mb_init(&bar[d], 1);
-        mb_fence_init();
-        while (issued < S64 - 1 && issued < total) issue();
-    }
-    __syncthreads();
-    if (total == 0) return;
-
-    if (warp == HELPER) {
-        StageCursor nx{0, 0};
-        LaneGeo G = lane_geo(a, tiles[0], lane);
-        FaceLane F = face_lane_bwd(a, G, lane, fJ, fK);
-        double fv[3] = {0.0, 0.0, 0.0};
-        auto load_faces = [&](int l) {
-            const double* sl = face_at(F, l, a.g.nx);
-#pragma unroll
-            for (int e = 0; e < 3; ++e) fv[e] = sl ? ld_relaxed(sl + e) : 0.0;
-        };
-        auto prepare = [&](long long g) {
-            double* sl = face_at(F, NL - 1 - nx.l, a.g.nx);
-            if (sl) take_slot(sl, fv, a.err);
-            if (F.hp >= 0) {
-                double* yb = ysh + (((int)(g & 1)) ^ 1) * YBUF + F.hp;
-                yb[0] = fv[0];
-                yb[YPL] = fv[1];
-                yb[2 * YPL] = fv[2];
-            }
-            advance(nx, NL);
-            if (g + 1 < total) {
-                if (nx.l == 0) {
-                    G = lane_geo(a, tiles[nx.m], lane);
-                    F = face_lane_bwd(a, G, lane, fJ, fK);
-                }
-                load_faces(NL - 1 - nx.l);
-            }
-        };
-        load_faces(NL - 1);
-        long long g = 0;
-        for (int m = 0; m < ntiles; ++m) {   // first stage of a tile: as in the forward sweep
-            prepare(g);
-            __syncthreads();
-            for (int step = 0; step < NL; ++step, ++g) {
-                if (lane == 0 && issued < total) issue();
-                if (step + 1 < NL) prepare(g + 1);
-                __syncthreads();
-            }
-        }
-        return;
-    }
-
-    const int rw = warp;
-    const int op = kk * HJ + jj;   // interior at [kk][jj], borders at row TK and column TJ
-    long long g = 0;
-    for (int m = 0; m < ntiles; ++m) {
+        for (int q = threadIdx.x; q < 2 * SLOT; q += SWEEP_THREADS) ex[PLANE + q] = 0.0;
+        for (int q = threadIdx.x; q < SLOT; q += SWEEP_THREADS) ex[ZERO + q] = 0.0;
         __syncthreads();
-        const LaneGeo G = lane_geo(a, tiles[m], lane);
-        const bool feedJ = G.valid && jj == 0 && G.J > 0 && !ycut(a, G.J * TJ);
-        const bool feedK = G.valid && kk == 0 && G.K > 0 && !zcut(a, G.K * TK);
-        double* fjo = fJ + jslot(a, G.t, 0, kk, 3) + rw - (size_t)G.l0 * TK * 3;
-        double* fko = fK + kslot(a, G.t, 0, jj, 3) + rw - (size_t)G.l0 * TJ * 3;
-        double* zo = z + (size_t)rw * n + G.cbase;
-        for (int step = 0; step < NL; ++step, ++g) {
-            const int l = NL - 1 - step;
-            const int st = (int)(g % S64);
-            mb_wait(&bar[st], (unsigned)((g / S64) & 1), a.err);
-            const double* U = ring + (size_t)st * STAGE + 3 * rw * 32 + lane;
-            const double* yb = ysh + (((int)(g & 1)) ^ 1) * YBUF + op;
-            // three independent chains (y and the +x block, the +y block, the +z
-            // block), then two adds
-            double u = ring[(size_t)st * STAGE + (BLK_ENT + rw) * 32 + lane];
-            double v = -U[9 * 32] * yb[1];
-            double w = -U[18 * 32] * yb[HJ];
-#pragma unroll
-            for (int s2 = 0; s2 < 3; ++s2) u = fma(-U[s2 * 32], yb[s2 * YPL], u);            // +x
-#pragma unroll
-            for (int s2 = 1; s2 < 3; ++s2) v = fma(-U[(9 + s2) * 32], yb[s2 * YPL + 1], v);   // +y
-#pragma unroll
-            for (int s2 = 1; s2 < 3; ++s2) w = fma(-U[(18 + s2) * 32], yb[s2 * YPL + HJ], w); // +z
-            const bool act = lane_active(a, G, l);
-            const double acc = act ? u + (v + w) : 0.0;
-            ysh[(int)(g & 1) * YBUF + rw * YPL + op] = acc;
-            if (act) {
-                zo[l] = acc;
-                if (feedJ) st_relaxed(fjo + (size_t)l * TK * 3, acc);
-                if (feedK) st_relaxed(fko + (size_t)l * TJ * 3, acc);
+        const unsigned rank = s_rank;
+        if (rank >= (unsigned)a.T) return;   // every CTA draws exactly one ticket past the end
+        const SweepTile t = a.tiles[rank];
+        // parity of level l's mbarrier phase: the uses of its place so far
+        auto parity = [&](int l) {
+            const int uses = (NL - (l & (RING - 1)) + RING - 1) / RING;
+            return (unsigned)(turn * uses + l / RING) & 1u;
+        };
+
+        if (warp == TSJ + FACE_WARPS) {
+            // ---- copy warp: a level's factors and right-hand side into its place,
+            // once the level that held it before has begun (its entries are read
+            // one level earlier) ------------------------------------------------
+            if (lane == 0) {
+                const double* Sp = S + (size_t)rank * NL * (TSJ * 96);
+                const double* Qp = Q + (size_t)rank * NL * SLOT;
+                for (int l = 0; l < NL; ++l) {
+                    int q = 0;
+                    while (ld_level(&s_done) + RING < l + 1 && ++q < WAIT_LIMIT) __nanosleep(20);
+                    if (q >= WAIT_LIMIT) atomicExch(a.err, 1);
+                    unsigned long long* b = &bar[l & (RING - 1)];
+                    double* dst = ring[l & (RING - 1)];
+                    mb_expect(b, STAGE * 8);
+                    bulk_g2s(dst, Sp + (size_t)l * (TSJ * 96), TSJ * 96 * 8, b);
+                    bulk_g2s(dst + TSJ * 96, Qp + (size_t)l * SLOT, SLOT * 8, b);
+                }
             }
-            __syncthreads();
+        } else if (warp >= TSJ) {
+            // ---- face warps: levels warp - TSJ, + FACE_WARPS, ... ------------
+            const bool jf = lane < 3 * TSK;
+            const int e = jf ? lane : lane - 3 * TSK;
+            const int line = e / 3, comp = e % 3;
+            const bool has = lane < FACE_LANES && (jf ? t.depJ && line < t.nk : t.depK && line < t.nj);
+            double* in = a.inbox + (size_t)rank * NL * FACE_W + lane;
+            const int to = HALO + comp * LINES + (jf ? line : TSK + line);
+            const double sent = __longlong_as_double((long long)SENTINEL_BITS);
+            bool abort = false;
+            int q = 0;
+            // the later levels are polled once the first has come
+            while (warp > TSJ && ld_level(&s_begun) == 0 && ++q < WAIT_LIMIT) __nanosleep(32);
+            for (int l = warp - TSJ; l < NL; l += FACE_WARPS) {
+                // the ring place was read at level l - RING
+                for (q = 0; ld_level(&s_done) + RING <= l && q < WAIT_LIMIT; ++q) __nanosleep(32);
+                if (q == WAIT_LIMIT && lane == 0) atomicExch(a.err, 1);
+                const int i = l - line;
+                const bool need = has && i >= 0 && i < nx;
+                double* at = in + (size_t)l * FACE_W;
+                double v = need ? ld_relaxed(at) : 0.0;
+                for (q = 1; __any_sync(FULL, is_sentinel(v)) && !abort; ++q) {
+                    if (need) v = ld_relaxed(at);
+                    if ((q & 1023) == 0) {
+                        const bool late = q >= 4 * POLL_LIMIT;
+                        if (late && lane == 0) atomicExch(a.err, 1);
+                        abort = __any_sync(FULL, late || ld_relaxed_i(a.err) != 0);
+                    }
+                }
+                if (lane < FACE_LANES) ex[to + ((l + 1) & (RING - 1)) * SLOT] = is_sentinel(v) ? 0.0 : v;
+                if (l == 0 && lane == 0) st_level(&s_begun, 1);
+                // the next level's factors (the first one's too) are in
+                for (int m = l == 0 ? 0 : l + 1; m <= l + 1 && m < NL; ++m)
+                    for (q = 0; !__all_sync(FULL, mb_try(&bar[m & (RING - 1)], parity(m))); ++q)
+                        if (q >= WAIT_LIMIT / 16) {
+                            if (lane == 0) atomicExch(a.err, 1);
+                            break;
+                        }
+                __syncwarp();
+                level_arrive(l & (RING - 1));
+                if (need) st_relaxed(at, sent);
+            }
+        } else {
+            // ---- compute warps ----------------------------------------------
+            const bool work = lane < 27;
+            const int kk = work ? lane / 9 : TSK - 1, row = (lane % 9) / 3, d = lane % 3, jj = warp;
+            const bool valid = work && jj < t.nj && kk < t.nk;
+            const bool head = valid && d == 0;         // the lane that ends with the result
+            const bool rhs = work && d == 0;
+            // neighbour source at level l: src + ((l + 1) & mask) SLOT, components LINES apart
+            int src, mask;
+            if (d == 0) {
+                src = PLANE + kk * TSJ + jj;
+                mask = 1;
+            } else if (d == 1) {
+                src = jj > 0 ? PLANE + kk * TSJ + jj - 1 : t.depJ ? HALO + kk : ZERO;
+                mask = jj > 0 ? 1 : t.depJ ? RING - 1 : 0;
+            } else {
+                src = kk > 0 ? PLANE + (kk - 1) * TSJ + jj : t.depK ? HALO + TSK + jj : ZERO;
+                mask = kk > 0 ? 1 : t.depK ? RING - 1 : 0;
+            }
+            double L[3], q;                   // the current level's entries
+            const int mine = jj * 96 + lane, rhs_at = TSJ * 96 + (jj * TSK + kk) * 3 + row;
+            // where results go
+            const int l0 = jj + kk;
+            const int res = PLANE + row * LINES + kk * TSJ + jj;
+            double* outp = out;
+            long long ostep = 0;
+            double *pj = a.inbox, *pk = a.inbox;       // the neighbours' inboxes
+            bool toJ = false, toK = false;
+            if (head) {
+                if (FWD) {
+                    const int jk = (t.j0 + jj) + a.g.ny * (t.k0 + kk);
+                    ostep = -(long long)SLOT;
+                    outp = out + (size_t)lbout[jk] + row - (long long)(l0 + 1) * ostep;
+                } else {
+                    const int j = a.g.ny - 1 - (t.j0 + jj), k = a.g.nz - 1 - (t.k0 + kk);
+                    ostep = -1;
+                    outp = out + (size_t)row * n + (size_t)nx * (j + (size_t)a.g.ny * k) + (nx - 1) + l0 + 1;
+                }
+                toJ = t.nextJ >= 0 && jj == TSJ - 1;
+                toK = t.nextK >= 0 && kk == TSK - 1;
+                if (toJ) pj = a.inbox + ((long long)t.nextJ * NL - (TSJ - 1)) * FACE_W + kk * 3 + row;
+                if (toK) pk = a.inbox + ((long long)t.nextK * NL - (TSK - 1)) * FACE_W + 3 * TSK + jj * 3 + row;
+            }
+            double acc = 0.0;                 // the last level's result, not yet written out
+            bool act = false;
+            int ya = src + (1 & mask) * SLOT;
+            unsigned i = (unsigned)-l0;       // this level's cell of the line
+            for (int lb = 0; lb < NL; lb += RING) {
+#pragma unroll
+                for (int u = 0; u < RING; ++u) {
+                    const int l = lb + u;
+                    if (l >= NL) break;
+                    level_sync(u);
+                    const double y0 = ex[ya], y1 = ex[ya + LINES], y2 = ex[ya + 2 * LINES];
+                    if (u == 0 && l == 0) {
+#pragma unroll
+                        for (int s = 0; s < 3; ++s) L[s] = ring[0][mine + s * 32];
+                        q = rhs ? ring[0][rhs_at] : -0.0;   // the other chains start from nothing
+                    }
+                    double v = fma(-L[0], y0, q);
+                    v = fma(-L[1], y1, v);
+                    v = fma(-L[2], y2, v);
+                    // in the shadow of the chain: the last level's result, the next
+                    // level's entries
+                    if (act) *outp = acc;
+                    outp += ostep;
+                    if (threadIdx.x == 0) st_level(&s_done, l);
+#pragma unroll
+                    for (int s = 0; s < 3; ++s) L[s] = ring[(u + 1) % RING][mine + s * 32];
+                    q = rhs ? ring[(u + 1) % RING][rhs_at] : -0.0;
+                    const bool in = i < (unsigned)nx;
+                    act = in && head;
+                    ++i;
+                    ya = src + ((l + 2) & mask) * SLOT;
+                    // u + (v + w): the j-1 lane adds the k-1 chain, the i-1 lane the sum
+                    const double vw = v + __shfl_down_sync(FULL, v, 1);
+                    acc = v + __shfl_down_sync(FULL, vw, 1);
+                    if (!(in && valid)) acc = 0.0;
+                    if (rhs) ex[res + (u & 1) * SLOT] = acc;
+                    if (in && toJ) st_relaxed(pj, acc);
+                    if (in && toK) st_relaxed(pk, acc);
+                    pj += FACE_W;
+                    pk += FACE_W;
+                }
+            }
+            if (act) *outp = acc;
         }
+        __syncthreads();   // the plane, the rings and the ticket are free again
     }
 }
 
 // ---------------------------------------------------------------------------
-// Host side
+// Host side: tiles of both directions
 // ---------------------------------------------------------------------------
-constexpr size_t SWEEP_SMEM = sizeof(double) * (S64 * STAGE + 2 * YBUF) +
-                              sizeof(unsigned long long) * S64 + sizeof(int) * MAX_CTA_TILES;
-
-// Tiles in the order a wavefront reaches them: the level at which tile
-// (J, K) can start is TJ (J - J0) + TK (K - K0) within its block-Jacobi box
-// (J0, K0: the box's first tile), ties by (K, J).  Every dependency of a tile
-// (J - 1, K), (J, K - 1) in the same box comes earlier in the list.
-std::vector<int> sweep_tile_order(const TileArgs& a) {
-    const int bj = a.ysub > 0 ? a.ysub / TJ : a.NJ, bk = a.zsub > 0 ? a.zsub / TK : a.NK;
-    std::vector<int> t(a.T);
-    for (int q = 0; q < a.T; ++q) t[q] = q;
-    auto key = [&](int q) {
-        const int J = q % a.NJ, K = q / a.NJ;
-        return std::make_tuple(TJ * (J % bj) + TK * (K % bk), K, J);
-    };
-    std::sort(t.begin(), t.end(), [&](int x, int y) { return key(x) < key(y); });
+namespace {
+// The tiles of one axis: boxes of `sub` lines (0: one box) counted from the
+// low end of the grid, cut into tiles of `ext` lines from each box's first
+// line in the sweep's direction.
+struct AxisTile {
+    int start, count, box;   // box: first line of its box
+    bool dep;                // depends on the tile before it
+};
+std::vector<AxisTile> axis_tiles(int n, int sub, int ext, bool mirrored) {
+    std::vector<std::pair<int, int>> boxes;   // [begin, end) in the sweep's direction
+    const int step = sub > 0 ? sub : n;
+    for (int b = 0; b < n; b += step) {
+        const int e = std::min(n, b + step);
+        boxes.emplace_back(mirrored ? n - e : b, mirrored ? n - b : e);
+    }
+    std::sort(boxes.begin(), boxes.end());
+    std::vector<AxisTile> t;
+    for (const auto& x : boxes)
+        for (int s = x.first; s < x.second; s += ext)
+            t.push_back({s, std::min(ext, x.second - s), x.first, s > x.first});
     return t;
 }
+}  // namespace
 
-// Persistent CTAs of the sweeps: sweep_ctas_per_sm per SM (1 or 2; with two,
-// the row warps of the two CTAs share the SM sub-partitions' FP64 pipes).
-int sweep_ctas(const bo_sim* s) {
+SweepOrder sweep_order(const Geom& g, int ysub, int zsub, bool mirrored) {
+    const std::vector<AxisTile> tj = axis_tiles(g.ny, ysub, TSJ, mirrored);
+    const std::vector<AxisTile> tk = axis_tiles(g.nz, zsub, TSK, mirrored);
+    const int NJ = (int)tj.size(), NK = (int)tk.size(), T = NJ * NK, NL = g.nx + TSJ + TSK - 2;
+    // topological order: the level at which a tile can start within its box
+    std::vector<int> ids(T), rank(T);
+    for (int q = 0; q < T; ++q) ids[q] = q;
+    auto key = [&](int q) {
+        const AxisTile &a = tj[q % NJ], &b = tk[q / NJ];
+        return std::make_tuple((a.start - a.box) + (b.start - b.box), q);
+    };
+    std::sort(ids.begin(), ids.end(), [&](int x, int y) { return key(x) < key(y); });
+    for (int q = 0; q < T; ++q) rank[ids[q]] = q;
+    SweepOrder o;
+    o.T = T;
+    o.tiles.resize(T);
+    o.line.assign((size_t)g.ny * g.nz, 0);
+    for (int J = 0; J < NJ; ++J)
+        for (int K = 0; K < NK; ++K) {
+            const int r = rank[J + NJ * K];
+            SweepTile& t = o.tiles[r];
+            t.j0 = tj[J].start;
+            t.k0 = tk[K].start;
+            t.nj = (short)tj[J].count;
+            t.nk = (short)tk[K].count;
+            t.depJ = tj[J].dep;
+            t.depK = tk[K].dep;
+            t.nextJ = J + 1 < NJ && tj[J + 1].dep ? rank[J + 1 + NJ * K] : -1;
+            t.nextK = K + 1 < NK && tk[K + 1].dep ? rank[J + NJ * (K + 1)] : -1;
+            for (int jj = 0; jj < t.nj; ++jj)
+                for (int kk = 0; kk < t.nk; ++kk) {
+                    const int j = mirrored ? g.ny - 1 - (t.j0 + jj) : t.j0 + jj;
+                    const int k = mirrored ? g.nz - 1 - (t.k0 + kk) : t.k0 + kk;
+                    const size_t lev = (size_t)r * NL + jj + kk + (mirrored ? g.nx - 1 : 0);
+                    o.line[j + (size_t)g.ny * k] = (unsigned)(lev * SLOT + (jj * TSK + kk) * 3);
+                }
+        }
+    return o;
+}
+
+SweepArgs sweep_args(const bo_sim* s, int dir) {
+    const SweepPlan& p = s->sweep;
+    SweepArgs a;
+    a.g = s->geo;
+    a.T = p.T;
+    a.NL = p.NL;
+    a.tiles = p.tiles[dir];
+    a.inbox = p.inbox;
+    a.ticket = p.ticket + dir;
+    a.err = s->d_sweep_sync + 2;
+    return a;
+}
+
+SweepFactors sweep_factors(const bo_sim* s) {
+    const SweepPlan& p = s->sweep;
+    return SweepFactors{p.line[0], p.line[1], p.S[0], p.S[1], p.Dn};
+}
+
+// CTAs of a sweep per SM: sweep_ctas_per_sm (two by default).  Up to 470 tiles
+// (3 an SM) could be under way in the middle of the 60x220x85 model's
+// wavefront, but tiles on one SM share its FP64 pipes (one warp instruction in
+// 19 cycles, 20 a tile level): 2, 3 and 4 CTAs per SM took 265, 276 and 288 us.
+static int sweep_grid(const bo_sim* s) {
     int dev, sms;
     BO_CUDA(cudaGetDevice(&dev));
     BO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    return std::min(tile_args(s).T, s->sweep_ctas_per_sm * sms);
+    return std::min(s->sweep.T, s->sweep_ctas_per_sm * sms);
 }
 
+static void free_plan(SweepPlan& p) {
+    void* ptrs[] = {p.tiles[0], p.tiles[1], p.line[0], p.line[1], p.S[0], p.S[1],
+                    p.Q[0],     p.Q[1],     p.inbox,   p.ticket,  p.Dn};
+    for (void* q : ptrs)
+        if (q) cudaFree(q);
+    p = SweepPlan();
+}
+void free_sweeps64(bo_sim* s) { free_plan(s->sweep); }
+
+__global__ void k_fill_inbox(double* __restrict__ p, size_t count) {
+    const double sent = __longlong_as_double((long long)SENTINEL_BITS);
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < count;
+         q += (size_t)gridDim.x * blockDim.x)
+        p[q] = sent;
+}
+void reset_inbox(bo_sim* s, cudaStream_t st) {
+    const SweepPlan& p = s->sweep;
+    k_fill_inbox<<<304, 256, 0, st>>>(p.inbox, (size_t)p.T * p.NL * FACE_W);
+    count_launch(s, st);
+    BO_LAUNCH_CHECK("k_fill_inbox");
+}
+
+// The tickets of a launch are counted from the last launch's with the same grid.
+void reset_tickets(bo_sim* s) {
+    BO_CUDA(cudaMemset(s->sweep.ticket, 0, 2 * sizeof(unsigned long long)));
+}
+
+// Plan of both sweeps for the current block-Jacobi boxes.  The new plan is
+// complete before the old one is given up.
 void setup_sweeps64(bo_sim* s) {
-    BO_CUDA(cudaFuncSetAttribute(k_fwd64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM));
-    BO_CUDA(cudaFuncSetAttribute(k_bwd64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM));
-    // two CTAs per SM need the whole shared-memory carveout
-    for (const void* k : {(const void*)k_fwd64, (const void*)k_bwd64})
+    const Geom& g = s->geo;
+    SweepPlan p;
+    try {
+        p.NL = g.nx + TSJ + TSK - 2;
+        for (int d = 0; d < 2; ++d) {
+            const SweepOrder o = sweep_order(g, s->ysub, s->zsub, d == 1);
+            p.T = o.T;
+            const size_t lev = (size_t)o.T * p.NL;
+            if (lev * SLOT >= (1ull << 32))
+                fail(BO_ERR_INVALID_ARG, "grid too large for the sweeps' 32-bit positions");
+            auto alloc = [&](auto** q, size_t count) {
+                BO_CUDA(cudaMalloc(reinterpret_cast<void**>(q), sizeof(**q) * count));
+                BO_CUDA(cudaMemset(*q, 0, sizeof(**q) * count));   // idle slots stay zero
+            };
+            alloc(&p.tiles[d], o.tiles.size());
+            alloc(&p.line[d], o.line.size());
+            alloc(&p.S[d], lev * TSJ * 96);
+            alloc(&p.Q[d], lev * SLOT);
+            BO_CUDA(cudaMemcpy(p.tiles[d], o.tiles.data(), sizeof(SweepTile) * o.tiles.size(),
+                               cudaMemcpyHostToDevice));
+            BO_CUDA(cudaMemcpy(p.line[d], o.line.data(), sizeof(unsigned) * o.line.size(),
+                               cudaMemcpyHostToDevice));
+            if (d == 0) {
+                alloc(&p.inbox, lev * FACE_W);
+                alloc(&p.ticket, 2);
+                alloc(&p.Dn, 9 * (size_t)g.n);
+            }
+        }
+    } catch (...) {
+        free_plan(p);
+        throw;
+    }
+    free_plan(s->sweep);
+    s->sweep = p;
+    // four CTAs on an SM need 144 KB of shared memory
+    for (const void* k : {(const void*)k_sweep<true>, (const void*)k_sweep<false>})
         BO_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared));
-    int dev, sms, pf = 0, pb = 0;
-    BO_CUDA(cudaGetDevice(&dev));
-    BO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    BO_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pf, k_fwd64, SW_THREADS, SWEEP_SMEM));
-    BO_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pb, k_bwd64, SW_THREADS, SWEEP_SMEM));
-    if ((long long)std::min(pf, pb) * sms < sweep_ctas(s))
-        fail(BO_ERR_INVALID_ARG, "sweep CTAs cannot all be resident at once");
-    const TileArgs a = tile_args(s);
-    if ((a.T + sweep_ctas(s) - 1) / sweep_ctas(s) > MAX_CTA_TILES)
-        fail(BO_ERR_INVALID_ARG, "grid too large: more wavefront tiles per CTA than the sweeps hold");
-    update_sweep_order(s);
-}
-
-// Tile lists of both directions for the current block-Jacobi boxes.
-void update_sweep_order(bo_sim* s) {
-    const TileArgs a = tile_args(s);
-    std::vector<int> f = sweep_tile_order(a);
-    std::vector<int> both(2 * (size_t)a.T);
-    for (int q = 0; q < a.T; ++q) {
-        both[q] = f[q];
-        both[a.T + q] = f[a.T - 1 - q];
-    }
-    BO_CUDA(cudaMemcpy(s->d_order, both.data(), sizeof(int) * both.size(), cudaMemcpyHostToDevice));
+    reset_inbox(s, s->stream);
+    BO_CUDA(cudaStreamSynchronize(s->stream));
 }
 
 void enqueue_fwd64(bo_sim* s, cudaStream_t st, const double* r, const KrylovScalars* ks) {
-    SweepArgs A{tile_args(s), s->d_order, sweep_ctas(s)};
-    k_q_tiles<<<152 * 8, 256, 0, st>>>(A.a, (const double*)s->d_P, r, s->d_qt, ks);
+    const SweepPlan& p = s->sweep;
+    k_sweep_rhs<<<152 * 8, 256, 0, st>>>(s->geo.n, s->geo.nx, p.line[0], p.Dn, r, p.Q[0], ks);
     count_launch(s, st);
-    launch_coop_smem(st, A.G, SW_THREADS, SWEEP_SMEM, k_fwd64, A, (const double*)s->d_P,
-                     (const double*)s->d_qt, s->d_yt, faceJ3(s), faceK3(s), ks);
+    k_sweep<true><<<sweep_grid(s), SWEEP_THREADS, 0, st>>>(sweep_args(s, 0), p.S[0], p.Q[0],
+                                                           p.line[1], p.Q[1], ks);
     count_launch(s, st);
+    BO_LAUNCH_CHECK("k_sweep forward");
 }
 
 void enqueue_bwd64(bo_sim* s, cudaStream_t st, double* z, const KrylovScalars* ks) {
-    SweepArgs A{tile_args(s), s->d_order + tile_args(s).T, sweep_ctas(s)};
-    launch_coop_smem(st, A.G, SW_THREADS, SWEEP_SMEM, k_bwd64, A, (const double*)s->d_P,
-                     (const double*)s->d_yt, z, faceJ3(s), faceK3(s), ks);
+    const SweepPlan& p = s->sweep;
+    k_sweep<false><<<sweep_grid(s), SWEEP_THREADS, 0, st>>>(sweep_args(s, 1), p.S[1], p.Q[1],
+                                                            nullptr, z, ks);
     count_launch(s, st);
+    BO_LAUNCH_CHECK("k_sweep backward");
 }
 
 }  // namespace bo

@@ -107,27 +107,37 @@ void launch_coop(cudaStream_t st, int grid, int block, void (*kern)(Args...), Ar
     BO_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
 }
 
-template <class... Args>
-void launch_coop_smem(cudaStream_t st, int grid, int block, size_t smem, void (*kern)(Args...),
-                      Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    BO_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
-}
-
-// FP64 sweeps (sweep64.cu)
-void setup_sweeps64(bo_sim* s);                              // attributes, residency, tile lists
+// FP64 sweeps (sweep64.cu): a CTA owns a tile of TSJ x TSK x-lines.  Tiles are
+// numbered in the order a sweep takes them (per direction), a tile has NL =
+// nx + TSJ + TSK - 2 levels, and position (tile NL + level) 36 + 3 (TSK jj + kk)
+// + row of Q holds a right-hand side entry.  S[((tile NL + level) TSJ + jj) 96
+// + 32 s + 9 kk + 3 row + d] is entry (row, s) of the scaled block towards
+// neighbour d.  line[j + ny k] is the Q position of cell (0, j, k); a step in i
+// is one level up (forward) or down (backward).
+constexpr int FACE_W = 24;   // doubles of a level in a tile's inbox: 9 j-face, 12 k-face
+struct SweepArgs {
+    Geom g;
+    int T, NL;
+    const SweepTile* tiles;
+    double* inbox;                // [T][NL][FACE_W] neighbours' values, sentinel until written
+    unsigned long long* ticket;   // tiles handed out; a launch takes T + grid of them
+    int* err;
+};
+struct SweepFactors {
+    const unsigned *fline, *bline;
+    double *F, *B, *Dn;           // S of both directions, D^-1 [9][n] in natural order
+};
+struct SweepOrder {
+    int T;
+    std::vector<SweepTile> tiles;
+    std::vector<unsigned> line;
+};
+SweepOrder sweep_order(const Geom& g, int ysub, int zsub, bool mirrored);
+SweepFactors sweep_factors(const bo_sim* s);
+void setup_sweeps64(bo_sim* s);                              // plan for the current boxes
+void reset_inbox(bo_sim* s, cudaStream_t st);
 void enqueue_fwd64(bo_sim* s, cudaStream_t st, const double* r, const KrylovScalars* ks);
 void enqueue_bwd64(bo_sim* s, cudaStream_t st, double* z, const KrylovScalars* ks);
-int sweep_ctas(const bo_sim* s);
 
 // FP32 sweeps of the mixed-precision solver (ilu_sweep32.cu)
 void setup_sweeps32(bo_sim* s);                              // attributes, residency check
