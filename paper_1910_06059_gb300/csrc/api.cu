@@ -150,7 +150,7 @@ static void learn_online_step(bo_sim* s) {
 // Offline set of the learned stage: free every kept system.
 void learn_set_clear(bo_sim* s) {
     for (LearnSystem& q : s->ml_set) {
-        void* ptrs[] = {q.A, q.P, q.featf, q.cell, q.r};
+        void* ptrs[] = {q.A, q.Dn, q.featf, q.cell, q.r};
         for (void* p : ptrs)
             if (p) cudaFree(p);
     }
@@ -166,16 +166,16 @@ static void learn_store_system(bo_sim* s) {
     BO_CUDA(cudaStreamSynchronize(s->stream));
     const int nr = std::min(cnt, s->ml_cap);
     if (nr <= 0) return;
-    const size_t n = s->geo.n, NA = 63 * n, NP = 63 * ilu_storage(s), NR = (size_t)nr * 3 * n;
+    const size_t n = s->geo.n, NA = 63 * n, ND = 9 * n, NR = (size_t)nr * 3 * n;
     LearnSystem q;
     bool ok = cudaMalloc(reinterpret_cast<void**>(&q.A), sizeof(double) * NA) == cudaSuccess &&
-              cudaMalloc(reinterpret_cast<void**>(&q.P), sizeof(double) * NP) == cudaSuccess &&
+              cudaMalloc(reinterpret_cast<void**>(&q.Dn), sizeof(double) * ND) == cudaSuccess &&
               cudaMalloc(reinterpret_cast<void**>(&q.featf), sizeof(float) * 64 * n) == cudaSuccess &&
               cudaMalloc(reinterpret_cast<void**>(&q.cell), sizeof(float4) * n) == cudaSuccess &&
               cudaMalloc(reinterpret_cast<void**>(&q.r), sizeof(double) * NR) == cudaSuccess;
     if (!ok) {
         (void)cudaGetLastError();   // the device is full: keep what was collected
-        void* ptrs[] = {q.A, q.P, q.featf, q.cell, q.r};
+        void* ptrs[] = {q.A, q.Dn, q.featf, q.cell, q.r};
         for (void* p : ptrs)
             if (p) cudaFree(p);
         s->ml_collect_max = (int)s->ml_set.size();
@@ -183,7 +183,7 @@ static void learn_store_system(bo_sim* s) {
     }
     q.nr = nr;
     BO_CUDA(cudaMemcpyAsync(q.A, s->d_A, sizeof(double) * NA, cudaMemcpyDeviceToDevice, s->stream));
-    BO_CUDA(cudaMemcpyAsync(q.P, s->d_P, sizeof(double) * NP, cudaMemcpyDeviceToDevice, s->stream));
+    BO_CUDA(cudaMemcpyAsync(q.Dn, s->sweep.Dn, sizeof(double) * ND, cudaMemcpyDeviceToDevice, s->stream));
     BO_CUDA(cudaMemcpyAsync(q.featf, s->d_ml_featf, sizeof(float) * 64 * n, cudaMemcpyDeviceToDevice,
                             s->stream));
     BO_CUDA(cudaMemcpyAsync(q.cell, s->d_ml_cell, sizeof(float4) * n, cudaMemcpyDeviceToDevice,
@@ -391,9 +391,6 @@ bo_status bo_create_grid(int nx, int ny, int nz, const double* dx, const double*
             dalloc(&s->d_props, (size_t)NPROP * n);
             dalloc(&s->d_R, 3 * n);
             dalloc(&s->d_A, 63 * n);
-            dalloc(&s->d_P, 63 * ilu_storage(s));
-            // idle slots of the tile order are never written: zero factors
-            BO_CUDA(cudaMemset(s->d_P, 0, sizeof(double) * 63 * ilu_storage(s)));
             dalloc(&s->d_face, face_storage(s));
             dalloc(&s->d_sweep_sync, 4);
             for (double** v : {&s->d_b, &s->d_xs, &s->d_r, &s->d_rh, &s->d_pk, &s->d_v, &s->d_s,
@@ -948,7 +945,11 @@ bo_status bo_set_precision(bo_sim* s, int precision) {
             dalloc(&s->d_y32, vec32_floats(s));
         }
         s->mixed = mixed;
-        if (mixed) convert_factors32(s, s->stream);  // factors of an earlier bo_factor stay usable
+        if (mixed) {   // factors of an earlier bo_factor stay usable
+            need_tile_factors(s);
+            enqueue_tile_factors(s, s->stream);
+            convert_factors32(s, s->stream);
+        }
         reset_sweep_faces(s);
         build_graphs(s);
         sync(s);
@@ -1148,29 +1149,29 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
         const size_t N = 3 * (size_t)s->geo.n;
         double first = 0.0, last = 0.0;
         long long cnt = 0;
-        // each kept system's Jacobian, ILU(0) data, features and scalings take
+        // each kept system's Jacobian, pivot inverses, features and scalings take
         // the place of the current ones while its residuals are trained on
         struct Swap {
             bo_sim* s;
-            double *A, *P;
+            double *A, *Dn;
             float* featf;
             float4* cell;
             ~Swap() {
                 s->d_A = A;
-                s->d_P = P;
+                s->sweep.Dn = Dn;
                 s->d_ml_featf = featf;
                 s->d_ml_cell = cell;
             }
         };
         {
-        Swap keep{s, s->d_A, s->d_P, s->d_ml_featf, s->d_ml_cell};
+        Swap keep{s, s->d_A, s->sweep.Dn, s->d_ml_featf, s->d_ml_cell};
         for (int ep = 0; ep < epochs; ++ep) {
             for (const LearnSystem& q : s->ml_set) {
                 s->d_A = q.A;
-                s->d_P = q.P;
+                s->sweep.Dn = q.Dn;
                 s->d_ml_featf = q.featf;
                 s->d_ml_cell = q.cell;
-                enqueue_factor_lower(s, s->stream);   // the sweeps' copies of its factors
+                enqueue_scaled_factors(s, s->stream);
                 for (int j = 0; j < q.nr; ++j) {
                     const double L = learn_loss_grad(s, q.r + (size_t)j * N);
                     if (ep == 0) first += L;
@@ -1182,7 +1183,7 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
             }
         }
         }
-        if (s->factored) enqueue_factor_lower(s, s->stream);
+        if (s->factored) enqueue_scaled_factors(s, s->stream);
         sync(s);
         check_timeout(s);
         s->ml_train_ms +=
@@ -1311,6 +1312,10 @@ bo_status bo_set_solve_schedule(bo_sim* s, int kind) {
         need(kind == BO_SCHEDULE_TILED || kind == BO_SCHEDULE_BLOCK, BO_ERR_INVALID_ARG,
              "bo_set_solve_schedule: kind must be BO_SCHEDULE_TILED or BO_SCHEDULE_BLOCK");
         s->solve_schedule = kind;
+        if (kind == BO_SCHEDULE_BLOCK && s->factored) {
+            need_tile_factors(s);
+            enqueue_tile_factors(s, s->stream);
+        }
     });
 }
 

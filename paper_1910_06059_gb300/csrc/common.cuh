@@ -32,8 +32,9 @@ void check_cuda(cudaError_t e, const char* what, const char* file, int line);
 //   Jacobian A: 7 blocks per cell, block-major then entry-major:
 //     A[(b*9 + e)*n + c],  b: 0 diag, 1 -x, 2 +x, 3 -y, 4 +y, 5 -z, 6 +z,
 //     e = 3*r + s for dR_r,c / dy_s,neighbour(b); zero where no neighbour.
-//   ILU(0) data P in tile order (see tiles.cuh, pidx): b: 0 D^-1,
-//     1..3 D^-1 A_{c,-x/-y/-z}, 4..6 D^-1 A_{c,+x/+y/+z}.
+//   ILU(0): D^-1 [9][n] in natural order and the scaled blocks D^-1 A in the
+//     sweeps' lane orders (see tiles.cuh); P gathers them in the tile order of
+//     the FP32 sweeps and the one-CTA solve (pidx).
 // ---------------------------------------------------------------------------
 enum { NB_DIAG = 0, NB_MX = 1, NB_PX = 2, NB_MY = 3, NB_PY = 4, NB_MZ = 5, NB_PZ = 6 };
 constexpr int NPROP = 28;   // per-cell face quantities: rho_a, b_a lam_a (3 x 4), r_go b_o lam_o (4)
@@ -109,11 +110,11 @@ struct EagerTimer {
 };
 
 // One Newton system kept for offline training of the learned stage: its
-// Jacobian, ILU(0) data, FP32 features, per-cell scalings and nr residuals
+// Jacobian, pivot inverses, FP32 features, per-cell scalings and nr residuals
 // of its BiCGStab solve ([nr][3n]).
 struct LearnSystem {
     double* A = nullptr;
-    double* P = nullptr;
+    double* Dn = nullptr;
     float* featf = nullptr;
     float4* cell = nullptr;
     double* r = nullptr;
@@ -136,7 +137,8 @@ struct SweepPlan {
     double* S[2] = {nullptr, nullptr};      // scaled off-diagonal blocks, lane order
     double* Q[2] = {nullptr, nullptr};      // right-hand sides
     double* inbox = nullptr;
-    unsigned long long* ticket = nullptr;
+    double* inbox9 = nullptr;               // the factorisation's
+    unsigned long long* ticket = nullptr;   // forward, backward, factorisation
     double* Dn = nullptr;                   // D^-1 [9][n]
 };
 
@@ -182,7 +184,7 @@ struct bo_sim {
     double* d_props = nullptr;   // NPROP * n
     double* d_R = nullptr;       // 3n
     double* d_A = nullptr;       // 63n
-    double* d_P = nullptr;       // 63 x tile-order ILU(0) data
+    double* d_P = nullptr;       // 63 x tile-order ILU(0) data (FP32 sweeps, one-CTA solve; at need)
     bo::SweepPlan sweep;         // FP64 sweeps: tiles, factors, right-hand sides
     float* d_P32 = nullptr;      // FP32 factors in the FP32 sweep layout (mixed mode)
     float* d_r32 = nullptr;      // FP32 sweep input, tile order (mixed mode)
@@ -294,11 +296,12 @@ void launch_restore(bo_sim* s);
 
 void setup_sweeps(bo_sim* s);
 int sweep_timeout(bo_sim* s);
-size_t ilu_storage(const bo_sim* s);
 void setup_sweeps64(bo_sim* s);                  // FP64 sweep plan for the current boxes
 void free_sweeps64(bo_sim* s);
 void reset_tickets(bo_sim* s);                   // after a change of the sweeps' grid
-void enqueue_factor_lower(bo_sim* s, cudaStream_t st);   // scaled lower blocks, sweep copies
+void enqueue_scaled_factors(bo_sim* s, cudaStream_t st); // both sweeps' blocks from A and D^-1
+void need_tile_factors(bo_sim* s);               // the tile-order buffer d_P
+void enqueue_tile_factors(bo_sim* s, cudaStream_t st);   // gathers d_P from the factorisation
 size_t face_storage(const bo_sim* s);
 void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad);
 void enqueue_fwd(bo_sim* s, cudaStream_t st, const double* r, double* y, const KrylovScalars* ks);

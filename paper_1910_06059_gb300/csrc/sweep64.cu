@@ -22,7 +22,7 @@
 //   * A CTA has four such warps (one per sub-partition) and a tile of 4 x 3
 //     x-lines (TSJ x TSK); at tile level l, line (jj, kk) handles cell i = l - jj
 //     - kk.  Results pass through a small plane in shared memory, one barrier a
-//     level; a level of a tile on its own takes 619 cycles, 314 ns.
+//     level; a level of a tile on its own takes 600 cycles, 304 ns.
 //   * The factors are stored lane by lane, a level's 3 KB in one piece: a copy
 //     warp brings them and the right-hand side into a ring in shared memory with
 //     two bulk copies a level, RING levels ahead (cp.async by the compute warps
@@ -37,43 +37,24 @@
 //     level at which a tile can start).  A tile waits only for tiles with smaller
 //     tickets, which CTAs already running hold, so every wait ends whatever else
 //     shares the GPU and no launch has to be resident as a whole.
-// Measured, a sweep: 60x220x85 265 us (405 before, with one warp per row of an
-// 8 x 4 tile and a handoff per level), 33x27x9 31 us (52.6 before).
+// Measured, a sweep: 60x220x85 262 us (405 before, with one warp per row of an
+// 8 x 4 tile and a handoff per level), 33x27x9 30 us (52.6 before).
 // Waits are bounded; one that runs out sets the error flag and the sweep ends
 // with zeros for the missing values.
 #include <algorithm>
 #include <tuple>
 #include <vector>
 
-#include "tiles.cuh"
+#include "wavefront.cuh"
 
 namespace bo {
 
-constexpr int FACE_WARPS = 4;             // each opens every fourth level
-constexpr int SWEEP_THREADS = 32 * (TSJ + FACE_WARPS + 1);   // and the copy warp
-constexpr int WAIT_LIMIT = 1 << 26;       // polls of a level counter (several seconds)
-constexpr int LINES = TSJ * TSK;          // x-lines of a tile
-constexpr int RING = 8;                   // levels of the rings (power of two)
-constexpr int STAGE = 96 * TSJ + 3 * TSJ * TSK;   // doubles of a level: factors, right-hand side
+constexpr int SWEEP_THREADS = 32 * (TSJ + FACE_WARPS + 1);   // compute, face and copy warps
 constexpr int SLOT = 3 * LINES;           // doubles of one level in shared memory
+constexpr int STAGE = 96 * TSJ + SLOT;    // doubles of a level: factors, right-hand side
 constexpr int FACE_LANES = 3 * (TSK + TSJ);   // face values of one level: j-face, k-face
-static_assert(TSJ == 4 && TSK == 3, "one warp per j-line of the tile, three lines a warp");
 static_assert(TSJ + TSK <= LINES && FACE_LANES <= FACE_W, "a level's face values fit a slot");
 
-__device__ __forceinline__ unsigned sa(const void* p) {
-    return (unsigned)__cvta_generic_to_shared(p);
-}
-// Level counters in shared memory.  Plain volatile accesses: a warp's shared
-// memory accesses are performed in order, and a release would also wait for the
-// warp's global stores under way (several hundred cycles a level).
-__device__ __forceinline__ int ld_level(const int* p) {
-    int v;
-    asm volatile("ld.volatile.shared.b32 %0, [%1];" : "=r"(v) : "r"(sa(p)) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_level(int* p, int v) {
-    asm volatile("st.volatile.shared.b32 [%0], %1;" ::"r"(sa(p)), "r"(v) : "memory");
-}
 // mbarriers of the stages and the copies that complete them
 __device__ __forceinline__ void mb_init(unsigned long long* bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sa(bar)) : "memory");
@@ -101,17 +82,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
         "l"(src), "r"(bytes), "r"(sa(bar))
         : "memory");
 }
-// Opening of a level, on one of RING barriers in turn: its face warp arrives
-// (possibly several levels early), the compute warps wait.  The forms that
-// count threads: a warp that has come apart at a branch must not arrive twice.
-constexpr int OPEN = 32 * (TSJ + 1);
-__device__ __forceinline__ void level_sync(int place) {
-    asm volatile("barrier.cta.sync %0, %1;" ::"r"(1 + place), "n"(OPEN) : "memory");
-}
-__device__ __forceinline__ void level_arrive(int place) {
-    asm volatile("barrier.cta.arrive %0, %1;" ::"r"(1 + place), "n"(OPEN) : "memory");
-}
-
 // ---------------------------------------------------------------------------
 // q = D^-1 r in the forward sweep's order: its right-hand side, formed by all
 // SMs before the wavefront (9 products a cell, bound by bytes: 72 + 24 in, 24
@@ -164,14 +134,14 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
     }
     for (int turn = 0;; ++turn) {   // tiles this CTA has done
         if (threadIdx.x == 0) {
-            s_rank = (unsigned)(atomicAdd(a.ticket, 1ull) % (unsigned long long)(a.T + gridDim.x));
+            s_rank = draw_tile(a);
             s_done = s_begun = 0;
         }
         for (int q = threadIdx.x; q < 2 * SLOT; q += SWEEP_THREADS) ex[PLANE + q] = 0.0;
         for (int q = threadIdx.x; q < SLOT; q += SWEEP_THREADS) ex[ZERO + q] = 0.0;
         __syncthreads();
         const unsigned rank = s_rank;
-        if (rank >= (unsigned)a.T) return;   // every CTA draws exactly one ticket past the end
+        if (rank >= (unsigned)a.T) return;
         const SweepTile t = a.tiles[rank];
         // parity of level l's mbarrier phase: the uses of its place so far
         auto parity = [&](int l) {
@@ -211,22 +181,13 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
             // the later levels are polled once the first has come
             while (warp > TSJ && ld_level(&s_begun) == 0 && ++q < WAIT_LIMIT) __nanosleep(32);
             for (int l = warp - TSJ; l < NL; l += FACE_WARPS) {
-                // the ring place was read at level l - RING
-                for (q = 0; ld_level(&s_done) + RING <= l && q < WAIT_LIMIT; ++q) __nanosleep(32);
-                if (q == WAIT_LIMIT && lane == 0) atomicExch(a.err, 1);
+                await_place(&s_done, l, lane, a.err);
                 const int i = l - line;
-                const bool need = has && i >= 0 && i < nx;
-                double* at = in + (size_t)l * FACE_W;
-                double v = need ? ld_relaxed(at) : 0.0;
-                for (q = 1; __any_sync(FULL, is_sentinel(v)) && !abort; ++q) {
-                    if (need) v = ld_relaxed(at);
-                    if ((q & 1023) == 0) {
-                        const bool late = q >= 4 * POLL_LIMIT;
-                        if (late && lane == 0) atomicExch(a.err, 1);
-                        abort = __any_sync(FULL, late || ld_relaxed_i(a.err) != 0);
-                    }
-                }
-                if (lane < FACE_LANES) ex[to + ((l + 1) & (RING - 1)) * SLOT] = is_sentinel(v) ? 0.0 : v;
+                const bool need[1] = {has && i >= 0 && i < nx};
+                double* const at[1] = {in + (size_t)l * FACE_W};
+                double v[1];
+                poll_faces(at, need, v, abort, lane, a.err);
+                if (lane < FACE_LANES) ex[to + ((l + 1) & (RING - 1)) * SLOT] = v[0];
                 if (l == 0 && lane == 0) st_level(&s_begun, 1);
                 // the next level's factors (the first one's too) are in
                 for (int m = l == 0 ? 0 : l + 1; m <= l + 1 && m < NL; ++m)
@@ -237,7 +198,7 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
                         }
                 __syncwarp();
                 level_arrive(l & (RING - 1));
-                if (need) st_relaxed(at, sent);
+                if (need[0]) st_relaxed(at[0], sent);
             }
         } else {
             // ---- compute warps ----------------------------------------------
@@ -419,7 +380,7 @@ SweepFactors sweep_factors(const bo_sim* s) {
 // (3 an SM) could be under way in the middle of the 60x220x85 model's
 // wavefront, but tiles on one SM share its FP64 pipes (one warp instruction in
 // 19 cycles, 20 a tile level): 2, 3 and 4 CTAs per SM took 265, 276 and 288 us.
-static int sweep_grid(const bo_sim* s) {
+int sweep_grid(const bo_sim* s) {
     int dev, sms;
     BO_CUDA(cudaGetDevice(&dev));
     BO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -428,7 +389,7 @@ static int sweep_grid(const bo_sim* s) {
 
 static void free_plan(SweepPlan& p) {
     void* ptrs[] = {p.tiles[0], p.tiles[1], p.line[0], p.line[1], p.S[0], p.S[1],
-                    p.Q[0],     p.Q[1],     p.inbox,   p.ticket,  p.Dn};
+                    p.Q[0],     p.Q[1],     p.inbox,   p.inbox9,  p.ticket, p.Dn};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     p = SweepPlan();
@@ -445,12 +406,14 @@ void reset_inbox(bo_sim* s, cudaStream_t st) {
     const SweepPlan& p = s->sweep;
     k_fill_inbox<<<304, 256, 0, st>>>(p.inbox, (size_t)p.T * p.NL * FACE_W);
     count_launch(s, st);
+    k_fill_inbox<<<304, 256, 0, st>>>(p.inbox9, (size_t)p.T * p.NL * FACE9_W);
+    count_launch(s, st);
     BO_LAUNCH_CHECK("k_fill_inbox");
 }
 
 // The tickets of a launch are counted from the last launch's with the same grid.
 void reset_tickets(bo_sim* s) {
-    BO_CUDA(cudaMemset(s->sweep.ticket, 0, 2 * sizeof(unsigned long long)));
+    BO_CUDA(cudaMemset(s->sweep.ticket, 0, 3 * sizeof(unsigned long long)));
 }
 
 // Plan of both sweeps for the current block-Jacobi boxes.  The new plan is
@@ -480,7 +443,8 @@ void setup_sweeps64(bo_sim* s) {
                                cudaMemcpyHostToDevice));
             if (d == 0) {
                 alloc(&p.inbox, lev * FACE_W);
-                alloc(&p.ticket, 2);
+                alloc(&p.inbox9, lev * FACE9_W);
+                alloc(&p.ticket, 3);
                 alloc(&p.Dn, 9 * (size_t)g.n);
             }
         }

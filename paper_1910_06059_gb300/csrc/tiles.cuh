@@ -1,6 +1,6 @@
-// Tile schedule shared by the wavefront kernels (ILU(0) factorisation, the
-// FP64 sweeps and the FP32 sweeps): tile geometry, face slots, the sentinel
-// protocol of the face buffers and relaxed global accesses.
+// Tile geometry of the FP32 sweeps and the one-CTA solve (8 x 4 x-lines) and of
+// the FP64 wavefront kernels (4 x 3), face slots, the sentinel protocol of the
+// face buffers and relaxed global accesses.
 #pragma once
 #include "common.cuh"
 
@@ -115,6 +115,7 @@ void launch_coop(cudaStream_t st, int grid, int block, void (*kern)(Args...), Ar
 // neighbour d.  line[j + ny k] is the Q position of cell (0, j, k); a step in i
 // is one level up (forward) or down (backward).
 constexpr int FACE_W = 24;   // doubles of a level in a tile's inbox: 9 j-face, 12 k-face
+constexpr int FACE9_W = 64;  // the same for the factorisation's blocks: 27 j-face, 36 k-face
 struct SweepArgs {
     Geom g;
     int T, NL;
@@ -133,7 +134,9 @@ struct SweepOrder {
     std::vector<unsigned> line;
 };
 SweepOrder sweep_order(const Geom& g, int ysub, int zsub, bool mirrored);
+SweepArgs sweep_args(const bo_sim* s, int dir);
 SweepFactors sweep_factors(const bo_sim* s);
+int sweep_grid(const bo_sim* s);                             // CTAs of a wavefront launch
 void setup_sweeps64(bo_sim* s);                              // plan for the current boxes
 void reset_inbox(bo_sim* s, cudaStream_t st);
 void enqueue_fwd64(bo_sim* s, cudaStream_t st, const double* r, const KrylovScalars* ks);
