@@ -76,8 +76,8 @@ struct CprData {
     std::vector<CprLevel> lv;
     std::vector<std::vector<int>> h_agg;   // host copies of the aggregation maps
     int nc = 0;                            // size of the coarsest level
-    double* cwork = nullptr;               // [nc][2 nc] Gauss-Jordan work
-    double* cinv = nullptr;                // [nc][nc] inverse of the coarsest operator
+    double* cwork = nullptr;               // [nc][2 nc] Gauss-Jordan work (a large coarsest level)
+    double* cinv = nullptr;                // [nc][nc] inverse of the coarsest operator, by columns
     double* w = nullptr;                   // [3][n] quasi-IMPES weights
     double* x1 = nullptr;                  // [3][n] E_p x_p (components 1, 2 stay zero)
     double* r2 = nullptr;                  // [3][n] second-stage residual
@@ -233,6 +233,16 @@ static int l0_entry(int i, int j, const Geom& g) {
     return b * g.n + i;
 }
 
+// the inverse of the coarsest operator (below)
+constexpr int INV_CTAS = 16, INV_THREADS = 256, INV_MAX = 512;
+static size_t inv_smem(int nc) {
+    const size_t cols = (nc + INV_CTAS - 1) / INV_CTAS;
+    return sizeof(double) * (nc * cols + 2 * (nc + 2) + 2 * cols) + sizeof(int) * nc;
+}
+__global__ void k_cpr_coarse_inverse(Geom g0, int nc, const int* __restrict__ rowptr,
+                                     const int* __restrict__ colind, const double* __restrict__ val,
+                                     double* __restrict__ cinv, int* __restrict__ status);
+
 void cpr_build(bo_sim* s) {
     if (s->cpr) return;
     const Geom& g = s->geo;
@@ -325,7 +335,11 @@ void cpr_build(bo_sim* s) {
         }
     }
     c->nc = A[L - 1].n;
-    c->cwork = dzeros<double>((size_t)c->nc * 2 * c->nc);
+    if (c->nc > INV_MAX) c->cwork = dzeros<double>((size_t)c->nc * 2 * c->nc);
+    // opt-ins of the cluster kernel, attributes of the context
+    BO_CUDA(cudaFuncSetAttribute(k_cpr_coarse_inverse, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    BO_CUDA(cudaFuncSetAttribute(k_cpr_coarse_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)inv_smem(INV_MAX)));
     c->cinv = dzeros<double>((size_t)c->nc * c->nc);
     c->w = dzeros<double>(3 * (size_t)n);
     c->x1 = dzeros<double>(3 * (size_t)n);
@@ -421,10 +435,138 @@ __device__ __forceinline__ Nb7 nb7(const Geom& g, int c) {
     r.has[NB_PZ] = k + 1 < g.nz;
     return r;
 }
-// Coarsest operator to dense [A | I] and Gauss-Jordan with partial pivoting
-// by one CTA; the inverse lands in cinv.  A zero pivot sets status.
-__global__ void __launch_bounds__(1024)
+// Inverse of the coarsest operator by Gauss-Jordan with partial pivoting (the
+// largest |entry|, the first on ties), in place: a column that has been
+// eliminated holds the column of the inverse that its step brings in.  A zero
+// pivot sets status.  cinv is written transposed (column by column) for
+// k_cpr_coarse_apply.
+//
+// A cluster of INV_CTAS CTAs: nc steps of nc^2 products are 1.2 ms on the FP64
+// pipes of one SM at nc = 100 (with [A | I] in global memory the single CTA
+// before took 0.4 to 0.8 ms there and up to 5 ms at nc = 200, 1.3 ms on average in
+// an ensemble).  The columns are dealt out to the CTAs' shared memory, one thread
+// a row; the owner of step k's column finds the pivot and writes the column with
+// the pivot row exchanged into every CTA's buffer, and one cluster barrier a step
+// follows.  Measured: 179 us on the 61x58x15 member and 116 us on 60x110x43 (792
+// and 381 us before), 200 us on average in the ensemble (1,327 us).
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void st_cluster(double* p, int rank, double v) {
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+// size of |v| for the pivot search: ordered like |v|, a NaN counts as nothing
+__device__ __forceinline__ unsigned long long pivot_key(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+    return b > 0x7FF0000000000000ull ? 0ull : b;
+}
+__global__ void __launch_bounds__(INV_THREADS)
 k_cpr_coarse_inverse(Geom g0, int nc, const int* __restrict__ rowptr, const int* __restrict__ colind,
+                     const double* __restrict__ val, double* __restrict__ cinv,
+                     int* __restrict__ status) {
+    extern __shared__ double sm[];
+    const int cols = (nc + INV_CTAS - 1) / INV_CTAS;
+    double* M = sm;                            // [cols][nc]: column cl of this CTA is cl INV_CTAS + rank
+    double* bcast = M + (size_t)nc * cols;     // [2][nc + 2]: a step's column, 1 / pivot, pivot row
+    double* rowk = bcast + 2 * (nc + 2);       // [cols] the pivot row, scaled
+    double* rowp = rowk + cols;                // [cols] the row it replaces
+    int* orig = reinterpret_cast<int*>(rowp + cols);   // the matrix row now at each position
+    unsigned rank;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int mine = ((int)nc - (int)rank + INV_CTAS - 1) / INV_CTAS;   // columns of this CTA
+    for (int q = threadIdx.x; q < nc * cols; q += INV_THREADS) M[q] = 0.0;
+    for (int q = threadIdx.x; q < nc; q += INV_THREADS) orig[q] = q;
+    __syncthreads();
+    auto put = [&](int r, int c, double v) {
+        if (c % INV_CTAS == (int)rank) M[(size_t)(c / INV_CTAS) * nc + r] = v;
+    };
+    for (int r = threadIdx.x; r < nc; r += INV_THREADS) {
+        if (rowptr) {
+            for (int e = rowptr[r]; e < rowptr[r + 1]; ++e) put(r, colind[e], val[e]);
+        } else {   // the coarsest level is level 0: the 7-point layout val[b][n]
+            const Nb7 q = nb7(g0, r);
+            for (int b = 0; b < 7; ++b)
+                if (q.has[b]) put(r, q.nb[b], val[(size_t)b * nc + r]);
+        }
+    }
+    __shared__ int s_piv;
+    cluster_sync();   // every CTA has begun before another writes to it
+    for (int k = 0; k < nc; ++k) {
+        double* fb = bcast + (k & 1) * (nc + 2);
+        if (k % INV_CTAS == (int)rank) {       // this CTA holds column k
+            const double* col = M + (size_t)(k / INV_CTAS) * nc;
+            if (threadIdx.x < 32) {
+                unsigned long long best = 0;
+                int bi = nc;
+                for (int i = k + threadIdx.x; i < nc; i += 32) {
+                    const unsigned long long v = pivot_key(col[i]);
+                    if (bi == nc || v > best) {
+                        best = v;
+                        bi = i;
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const unsigned long long v = __shfl_down_sync(0xffffffffu, best, o);
+                    const int i = __shfl_down_sync(0xffffffffu, bi, o);
+                    if (v > best || (v == best && i < bi)) {
+                        best = v;
+                        bi = i;
+                    }
+                }
+                if (threadIdx.x == 0) {
+                    s_piv = bi;
+                    if (best == 0ull) *status = 1;
+                }
+            }
+            __syncthreads();
+            const int p = s_piv;
+            for (int i = threadIdx.x; i < nc + 2; i += INV_THREADS) {
+                const double v = i == nc ? 1.0 / col[p] : i == nc + 1 ? (double)p
+                                 : col[i == k ? p : i == p ? k : i];
+                for (int r = 0; r < INV_CTAS; ++r) st_cluster(fb + i, r, v);
+            }
+        }
+        cluster_sync();
+        const double inv = fb[nc];
+        const int p = (int)fb[nc + 1];
+        // the exchanged rows of this CTA's columns (the step's own column: that of
+        // the identity, 1 in row k)
+        for (int c = threadIdx.x; c < mine; c += INV_THREADS) {
+            const bool own = c * INV_CTAS + (int)rank == k;
+            rowk[c] = (own ? 1.0 : M[(size_t)c * nc + p]) * inv;
+            rowp[c] = own ? 0.0 : M[(size_t)c * nc + k];
+        }
+        if (threadIdx.x == 0) {
+            const int t = orig[k];
+            orig[k] = orig[p];
+            orig[p] = t;
+        }
+        __syncthreads();
+        const int ownc = k % INV_CTAS == (int)rank ? k / INV_CTAS : -1;
+        for (int i = threadIdx.x; i < nc; i += INV_THREADS) {
+            const double f = fb[i];
+            for (int c = 0; c < mine; ++c) {
+                double* m = M + (size_t)c * nc + i;
+                const double old = c == ownc ? 0.0 : i == p ? rowp[c] : *m;
+                *m = i == k ? rowk[c] : fma(-f, rowk[c], old);
+            }
+        }
+        __syncthreads();
+    }
+    for (int c = 0; c < mine; ++c) {
+        const int q = orig[c * INV_CTAS + (int)rank];
+        for (int i = threadIdx.x; i < nc; i += INV_THREADS) cinv[(size_t)q * nc + i] = M[(size_t)c * nc + i];
+    }
+    cluster_sync();   // no CTA leaves while another may still write to it
+}
+
+// The same in one CTA on [A | I] in global memory, for coarsest levels too large
+// for the cluster's shared memory (a hierarchy that stopped coarsening early).
+__global__ void __launch_bounds__(1024)
+k_cpr_coarse_inverse_large(Geom g0, int nc, const int* __restrict__ rowptr, const int* __restrict__ colind,
                      const double* __restrict__ val, double* __restrict__ M,
                      double* __restrict__ cinv, int* __restrict__ status) {
     const int m2 = 2 * nc;
@@ -501,7 +643,7 @@ k_cpr_coarse_inverse(Geom g0, int nc, const int* __restrict__ rowptr, const int*
         __syncthreads();
     }
     for (int q = threadIdx.x; q < nc * nc; q += blockDim.x) {
-        const int r = q / nc, col = q % nc;
+        const int col = q / nc, r = q % nc;
         cinv[q] = M[(size_t)r * m2 + nc + col];
     }
 }
@@ -664,17 +806,22 @@ k_cpr_sum(int nc, const int* __restrict__ mptr, const int* __restrict__ mem,
     }
 }
 
-// coarsest level: x = A^-1 b (dense)
-__global__ void __launch_bounds__(CPR_BS)
+// coarsest level: x = A^-1 b (dense), a row a thread in one chain over the
+// columns; cinv is stored by columns, so a warp's loads of a column are one piece,
+// and a block is one warp, so every chain has a sub-partition to itself (nc x 65
+// cycles; 256-thread blocks over the rows took 8 to 22 us).
+constexpr int CAP_BS = 32;
+__global__ void __launch_bounds__(CAP_BS)
 k_cpr_coarse_apply(int nc, const double* __restrict__ cinv, const double* __restrict__ b,
                    double* __restrict__ x, Prolong up, const KrylovScalars* __restrict__ ks) {
     if (ks != nullptr && ks->state != KS_RUN) return;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nc; r += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int q = 0; q < nc; ++q) s += cinv[(size_t)r * nc + q] * b[q];
-        x[r] = s;
-        prolong_row(up, r, s);
-    }
+    const int r = blockIdx.x * CAP_BS + threadIdx.x;
+    if (r >= nc) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int q = 0; q < nc; ++q) s = fma(cinv[(size_t)q * nc + r], b[q], s);
+    x[r] = s;
+    prolong_row(up, r, s);
 }
 
 // Second-stage residual r2 = r - S E_p x_p: only the pressure column of each
@@ -740,8 +887,25 @@ void enqueue_cpr_setup(bo_sim* s, cudaStream_t st) {
         count_launch(s, st);
     }
     const CprLevel& last = c->lv.back();
-    k_cpr_coarse_inverse<<<1, 1024, 0, st>>>(s->geo, c->nc, last.rowptr, last.colind, last.val,
-                                             c->cwork, c->cinv, c->status);
+    if (c->nc <= INV_MAX) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(INV_CTAS);
+        cfg.blockDim = dim3(INV_THREADS);
+        cfg.dynamicSmemBytes = inv_smem(c->nc);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = INV_CTAS;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        BO_CUDA(cudaLaunchKernelEx(&cfg, k_cpr_coarse_inverse, s->geo, c->nc, (const int*)last.rowptr,
+                                   (const int*)last.colind, (const double*)last.val, c->cinv,
+                                   c->status));
+    } else {
+        k_cpr_coarse_inverse_large<<<1, 1024, 0, st>>>(s->geo, c->nc, last.rowptr, last.colind,
+                                                       last.val, c->cwork, c->cinv, c->status);
+    }
     count_launch(s, st);
     BO_LAUNCH_CHECK("cpr setup");
 }
@@ -791,7 +955,8 @@ static void vcycle(bo_sim* s, cudaStream_t st, size_t l, const double* r,
             k_cpr_pre0<<<gr, CPR_BS, 0, st>>>(v.n, c->w, r, v.dinv, v.b, v.y, ks);
             count_launch(s, st);
         }
-        k_cpr_coarse_apply<<<gr, CPR_BS, 0, st>>>(v.n, c->cinv, v.b, v.x, up, ks);
+        k_cpr_coarse_apply<<<(v.n + CAP_BS - 1) / CAP_BS, CAP_BS, 0, st>>>(v.n, c->cinv, v.b, v.x,
+                                                                          up, ks);
         count_launch(s, st);
         return;
     }

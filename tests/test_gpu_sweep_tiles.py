@@ -1,8 +1,8 @@
-"""FP64 triangular sweeps at the edges of their tiles (4 x 3 x-lines, levels in
-rings of 8, a ticket per tile) against the oracle's ILU(0) apply, through the
-C ABI.
+"""Factorisation and FP64 triangular sweeps at the edges of their tiles (4 x 3 x-lines, levels in
+rings of 8, a ticket per tile) against the oracle's ILU(0), through the C ABI.
 
-Bar: 1e-10 of the vector's largest entry, as for the other applies on random
+Bars: pivot inverses 1e-8 per entry of their family (the conditioning argument of
+test_gpu_subdomains.py); applies 1e-10 of the vector's largest entry, as for the other applies on random
 states (two FP64 factorisations that sum in different orders differ by about
 cond(D) x 1.1e-16); a neighbour value that is missing, stale or taken from the
 wrong line gives errors of order one.  A repeated apply gives the same bits."""
@@ -13,7 +13,7 @@ import pytest
 
 import oracle
 import synth
-from helpers import vec_close
+from helpers import family_close, vec_close
 
 pytestmark = pytest.mark.gpu
 
@@ -58,8 +58,8 @@ def test_apply_at_tile_edges(shape, sub):
         s.set_state(*st)
         s.begin_step()
         s.assemble(2.0 * synth.DAY)
-    g.factor()
-    o.ilu0()
+    dinv = g.factor()
+    assert family_close(dinv, o.ilu0()[1], np.arange(o.n + 1), per_equation=False) <= 1e-8
     r = np.random.default_rng(11).normal(size=3 * g.n) * np.tile([1e-3, 1e-2, 1.0], g.n)
     z = g.precond_apply(r)
     assert vec_close(z, o.ilu_apply(r)) < 1e-10
