@@ -49,8 +49,12 @@ constexpr int CPR_GRID = 152 * 4;
 constexpr int CPR_GRID_ROWS = 152 * 8;   // coarse-level rows: latency-bound gathers, full occupancy
 // levels whose rows are short (the first coarse level: up to 32 entries, 12
 // on average) get an ELL copy and one thread per row; the longer rows of the
-// coarser levels are read by a warp per row
+// coarser levels are read by eight lanes per row
 constexpr int CPR_ELL_MAX = 32, CPR_ELL_AVG = 12;
+// ELL rows: entries whose loads are under way at once and blocks an SM (registers).
+// Measured per pass on 60x220x85's first coarse level: 22 us (4 and 6), 30 us (4
+// and 8), 25 us (8 and 4), 22 us (8 and 6), 37 us (16 and 3).
+constexpr int ELL_U = 4, ELL_BLOCKS = 6;
 
 struct CprLevel {
     int n = 0, nnz = 0;
@@ -703,78 +707,127 @@ struct Prolong {
     const int* mem = nullptr;
     double* xf = nullptr;
 };
-__device__ __forceinline__ void prolong_row(const Prolong& up, int I, double xI) {
+__device__ __forceinline__ void prolong_row(const Prolong& up, int I, double xI, int first = 0,
+                                            int step = 1) {
     if (up.xf == nullptr) return;
-    for (int q = up.mptr[I]; q < up.mptr[I + 1]; ++q) up.xf[up.mem[q]] += xI;
+    for (int q = up.mptr[I] + first; q < up.mptr[I + 1]; q += step) up.xf[up.mem[q]] += xI;
 }
 
-// Levels >= 1 in ELL form: one thread per row, the W entries of a row read
-// at e n + i (coalesced over the rows of a warp), all loads of a row
-// independent of each other.
+// Rows of the levels >= 1.
+//
+// ELL levels: one thread per row, the W entries of a row read at e n + i
+// (coalesced over the rows of a warp) and summed in order.  Padding (value 0)
+// takes no product: an FP64 warp instruction costs its SM 19 cycles, and rows
+// average under two thirds of W.
 __device__ __forceinline__ double ell_dot(int n, int W, int i, const int* __restrict__ col,
                                           const double* __restrict__ val,
                                           const double* __restrict__ x) {
+    constexpr int U = ELL_U;   // entries whose loads are under way at once
     double s = 0.0;
-    for (int e = 0; e < W; ++e) s += val[(size_t)e * n + i] * x[col[(size_t)e * n + i]];
+    for (int e0 = 0; e0 < W; e0 += U) {
+        double v[U], xj[U];
+        int c[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool in = e0 + u < W;
+            const size_t q = (size_t)(in ? e0 + u : 0) * n + i;
+            v[u] = val[q];
+            c[u] = col[q];
+            if (!in) v[u] = 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) xj[u] = x[c[u]];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (__double_as_longlong(v[u]) != 0) s = fma(v[u], xj[u], s);
+    }
     return s;
 }
+// Levels whose rows are long: ROW_LANES lanes per row over the CSR arrays.  The sum is
+// the tree of 32 strided partial sums (entries 32 apart in one chain, then pairs
+// 16, 8, 4, 2, 1 apart); a lane has four of the 32, so the first two steps stay in
+// it, and partial sums a short row leaves empty take no operation.  (A warp per
+// row, every step a shuffle, spent nine FP64 warp instructions a row; this
+// spends two to three: the three such levels of 60x220x85 took 21.7 us a
+// smoothing pass on average, 9.5 us now.)  All lanes of the group get here together; the result is in its
+// first lane.
+constexpr int ROW_LANES = 8;
+__device__ __forceinline__ double csr_dot(int i, bool active, const int* __restrict__ rowptr,
+                                          const int* __restrict__ colind,
+                                          const double* __restrict__ val,
+                                          const double* __restrict__ x) {
+    const int a = threadIdx.x & (ROW_LANES - 1);
+    double p[4] = {0.0, 0.0, 0.0, 0.0};
+    int len = 0;
+    if (active) {
+        const int e0 = rowptr[i];
+        len = rowptr[i + 1] - e0;
+        for (int t = 0; t < len; t += 32)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int e = t + 8 * m + a;
+                if (e < len) p[m] = fma(val[e0 + e], x[colind[e0 + e]], p[m]);
+            }
+    }
+    double s = p[0];
+    if (len > 16) s += p[2];
+    if (len > 8) s += len > 24 ? p[1] + p[3] : p[1];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, ROW_LANES);
+    return s;
+}
+// damped Jacobi's new value of a row
+__device__ __forceinline__ double jac_value(double x, double dinv, double b, double ax) {
+    return x + CPR_OMEGA * dinv * (b - ax);
+}
 
-// y = x + omega dinv (b - A x); with up, y is also added into the finer level
-__global__ void __launch_bounds__(CPR_BS)
-k_cpr_jac(int n, int W, const int* __restrict__ col, const double* __restrict__ val,
+// y = x + omega dinv (b - A x) (ROW_JAC; ROW_JAC_UP also adds y into the finer
+// level) or y = b - A x (ROW_RES), ELL
+enum { ROW_JAC = 0, ROW_RES = 1, ROW_JAC_UP = 2 };
+template <int MODE>
+__global__ void __launch_bounds__(CPR_BS, ELL_BLOCKS)
+k_cpr_ell(int n, int W, const int* __restrict__ col, const double* __restrict__ val,
           const double* __restrict__ dinv, const double* __restrict__ b,
           const double* __restrict__ x, double* __restrict__ y, Prolong up,
           const KrylovScalars* __restrict__ ks) {
     if (ks != nullptr && ks->state != KS_RUN) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double yi = x[i] + CPR_OMEGA * dinv[i] * (b[i] - ell_dot(n, W, i, col, val, x));
+        constexpr bool RES = MODE == ROW_RES;
+        const double bi = b[i], xi = RES ? 0.0 : x[i], di = RES ? 0.0 : dinv[i];   // ahead of the row
+        const double s = ell_dot(n, W, i, col, val, x);
+        const double yi = RES ? bi - s : jac_value(xi, di, bi, s);
         y[i] = yi;
-        prolong_row(up, i, yi);
+        if (MODE == ROW_JAC_UP) prolong_row(up, i, yi);
     }
 }
-
-// residual y = b - A x
+// The same over CSR rows.
+template <int MODE>
 __global__ void __launch_bounds__(CPR_BS)
-k_cpr_res(int n, int W, const int* __restrict__ col, const double* __restrict__ val,
+k_cpr_csr(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
+          const double* __restrict__ val, const double* __restrict__ dinv,
           const double* __restrict__ b, const double* __restrict__ x, double* __restrict__ y,
-          const KrylovScalars* __restrict__ ks) {
+          Prolong up, const KrylovScalars* __restrict__ ks) {
     if (ks != nullptr && ks->state != KS_RUN) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        y[i] = b[i] - ell_dot(n, W, i, col, val, x);
-}
-
-// Levels whose rows are long (the coarse ones): 32 lanes per row, the row's
-// entries strided over the lanes and summed by shuffles.  The loops run
-// warp-uniform so every lane reaches the shuffles.
-__device__ __forceinline__ double row_dot32(int i, bool active, int lane,
-                                            const int* __restrict__ rowptr,
-                                            const int* __restrict__ colind,
-                                            const double* __restrict__ val,
-                                            const double* __restrict__ x) {
-    double s = 0.0;
-    if (active)
-        for (int e = rowptr[i] + lane; e < rowptr[i + 1]; e += 32) s += val[e] * x[colind[e]];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    return s;
-}
-// y = x + omega dinv (b - A x) (RES = false) or y = b - A x (RES = true)
-template <bool RES>
-__global__ void __launch_bounds__(CPR_BS)
-k_cpr_csr32(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
-            const double* __restrict__ val, const double* __restrict__ dinv,
-            const double* __restrict__ b, const double* __restrict__ x, double* __restrict__ y,
-            Prolong up, const KrylovScalars* __restrict__ ks) {
-    if (ks != nullptr && ks->state != KS_RUN) return;
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int i = warp; i < n; i += nwarps) {   // warp-uniform
-        const double s = row_dot32(i, true, lane, rowptr, colind, val, x);
-        if (lane == 0) {
-            const double yi = RES ? b[i] - s : x[i] + CPR_OMEGA * dinv[i] * (b[i] - s);
-            y[i] = yi;
-            if (!RES) prolong_row(up, i, yi);
+    const int group = (blockIdx.x * blockDim.x + threadIdx.x) / ROW_LANES;
+    const int groups = gridDim.x * blockDim.x / ROW_LANES, first = group & ~(32 / ROW_LANES - 1);
+    for (int k = 0; first + k < n; k += groups) {   // warp-uniform
+        constexpr bool RES = MODE == ROW_RES;
+        const int i = group + k;
+        double bi = 0.0, xi = 0.0, di = 0.0;   // ahead of the row
+        if (i < n) {
+            bi = b[i];
+            if (!RES) {
+                xi = x[i];
+                di = dinv[i];
+            }
+        }
+        const int a = threadIdx.x % ROW_LANES;
+        const double s = csr_dot(i, i < n, rowptr, colind, val, x);
+        double yi = RES ? bi - s : jac_value(xi, di, bi, s);   // in the group's first lane
+        if (i < n && a == 0) y[i] = yi;
+        if (MODE == ROW_JAC_UP) {   // the group's lanes share the members
+            yi = __shfl_sync(0xffffffffu, yi, 0, ROW_LANES);
+            if (i < n) prolong_row(up, i, yi, a, ROW_LANES);
         }
     }
 }
@@ -910,31 +963,21 @@ void enqueue_cpr_setup(bo_sim* s, cudaStream_t st) {
     BO_LAUNCH_CHECK("cpr setup");
 }
 
-static int grid_for_rows(int n) {
-    return std::max(1, std::min(CPR_GRID_ROWS, (n + CPR_BS - 1) / CPR_BS));
+// short rows: one thread per row over the ELL copy; long rows: ROW_LANES lanes per
+// row over the CSR arrays
+static int grid_for_rows(const CprLevel& v) {
+    const int per = v.ell ? CPR_BS : CPR_BS / ROW_LANES;
+    return std::max(1, std::min(CPR_GRID_ROWS, (v.n + per - 1) / per));
 }
-// short rows (the first coarse level): one thread per row over the ELL copy;
-// long rows: a warp per row over the CSR arrays
-static int grid_warps(int n) {
-    return std::max(1, std::min(CPR_GRID_ROWS, (n + CPR_BS / 32 - 1) / (CPR_BS / 32)));
-}
-static void jac_ell(bo_sim* s, cudaStream_t st, const CprLevel& v, const double* x, double* y,
-                    const KrylovScalars* ks, Prolong up = Prolong{}) {
+template <int MODE>
+static void rows(bo_sim* s, cudaStream_t st, const CprLevel& v, const double* x, double* y,
+                 const KrylovScalars* ks, Prolong up = Prolong{}) {
     if (v.ell)
-        k_cpr_jac<<<grid_for_rows(v.n), CPR_BS, 0, st>>>(v.n, v.W, v.ecol, v.eval, v.dinv, v.b, x,
-                                                        y, up, ks);
+        k_cpr_ell<MODE><<<grid_for_rows(v), CPR_BS, 0, st>>>(v.n, v.W, v.ecol, v.eval, v.dinv, v.b, x,
+                                                           y, up, ks);
     else
-        k_cpr_csr32<false><<<grid_warps(v.n), CPR_BS, 0, st>>>(v.n, v.rowptr, v.colind, v.val,
-                                                              v.dinv, v.b, x, y, up, ks);
-    count_launch(s, st);
-}
-static void res_ell(bo_sim* s, cudaStream_t st, const CprLevel& v, const double* x, double* y,
-                    const KrylovScalars* ks) {
-    if (v.ell)
-        k_cpr_res<<<grid_for_rows(v.n), CPR_BS, 0, st>>>(v.n, v.W, v.ecol, v.eval, v.b, x, y, ks);
-    else
-        k_cpr_csr32<true><<<grid_warps(v.n), CPR_BS, 0, st>>>(v.n, v.rowptr, v.colind, v.val,
-                                                             v.dinv, v.b, x, y, Prolong{}, ks);
+        k_cpr_csr<MODE><<<grid_for_rows(v), CPR_BS, 0, st>>>(v.n, v.rowptr, v.colind, v.val, v.dinv,
+                                                           v.b, x, y, up, ks);
     count_launch(s, st);
 }
 
@@ -973,8 +1016,8 @@ static void vcycle(bo_sim* s, cudaStream_t st, size_t l, const double* r,
         k_cpr_res0<<<gr, CPR_BS, 0, st>>>(g, v.val, v.b, v.x, v.y, ks);
         count_launch(s, st);
     } else {   // the first sweep from zero came with the restriction into this level
-        jac_ell(s, st, v, v.y, v.x, ks);
-        res_ell(s, st, v, v.x, v.y, ks);
+        rows<ROW_JAC>(s, st, v, v.y, v.x, ks);
+        rows<ROW_RES>(s, st, v, v.x, v.y, ks);
     }
     k_cpr_sum<<<grid_for(w.n), CPR_BS, 0, st>>>(w.n, v.mptr, v.mem, v.y, w.b, w.dinv,
                                                w_coarsest ? nullptr : w.y, ks);
@@ -986,8 +1029,8 @@ static void vcycle(bo_sim* s, cudaStream_t st, size_t l, const double* r,
         k_cpr_jac0<<<gr, CPR_BS, 0, st>>>(g, v.val, v.dinv, v.b, v.y, v.x, ks);
         count_launch(s, st);
     } else {
-        jac_ell(s, st, v, v.x, v.y, ks);
-        jac_ell(s, st, v, v.y, v.x, ks, up);
+        rows<ROW_JAC>(s, st, v, v.x, v.y, ks);
+        rows<ROW_JAC_UP>(s, st, v, v.y, v.x, ks, up);
     }
 }
 
