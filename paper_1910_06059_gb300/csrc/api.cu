@@ -93,27 +93,30 @@ static void free_all(bo_sim* s) {
         if (p) cudaFree(p);
     if (s->h_ns) cudaFreeHost(s->h_ns);
     if (s->h_ks) cudaFreeHost(s->h_ks);
+    if (s->h_flags) cudaFreeHost(s->h_flags);
 }
 
 static void sync(bo_sim* s) { BO_CUDA(cudaStreamSynchronize(s->stream)); }
 
-static void read_status(bo_sim* s) {
+static void read_status(bo_sim* s, bool flags = false) {
     BO_CUDA(cudaMemcpyAsync(s->h_ns, s->d_ns, sizeof(NewtonStatus), cudaMemcpyDeviceToHost,
                             s->stream));
+    if (flags) read_flags_async(s);
     sync(s);
 }
 
-// Assembly plus the dead-well fix-up (one more assembly when a rate well has
-// no flowing connection), then the norms.
+// Assembly and norms, both once more after the dead-well fix-up when a rate well
+// has no flowing connection: one wait for the host in the usual case.
 static void assemble_and_norms(bo_sim* s, double dt) {
     launch_assemble(s, dt);
+    launch_norms(s, dt);
     read_status(s);
     if (s->h_ns->dead_wells > 0) {
         launch_fix_dead_wells(s);
         launch_assemble(s, dt);
+        launch_norms(s, dt);
+        read_status(s);
     }
-    launch_norms(s, dt);
-    read_status(s);
     s->assembled = true;
     s->factored = false;
     s->solved = false;
@@ -195,8 +198,9 @@ static void learn_store_system(bo_sim* s) {
 }
 
 // Linear solve of the last assembly; returns the LS_* status.
-static void check_timeout(bo_sim* s) {
-    if (sweep_timeout(s)) {
+// After a wait that followed read_flags_async.
+static void check_timeout_read(bo_sim* s) {
+    if (s->h_flags->sweep_timeout) {
         // leave the face buffers and the flag ready for the next call
         reset_sweep_faces(s);
         BO_CUDA(cudaMemsetAsync(s->d_sweep_sync + 2, 0, sizeof(int), s->stream));
@@ -205,11 +209,16 @@ static void check_timeout(bo_sim* s) {
              "a dataflow sweep gave up waiting for a neighbour (bounded wait ran out)");
     }
 }
+static void check_timeout(bo_sim* s) {
+    read_flags_async(s);
+    sync(s);
+    check_timeout_read(s);
+}
 
 static int solve_linear(bo_sim* s, double tol, int maxit, int* its) {
     launch_factor(s);
-    read_status(s);
-    check_timeout(s);
+    read_status(s, true);
+    check_timeout_read(s);
     if (s->h_ns->pad != 0) {  // non-finite pivot block
         *its = 0;
         return LS_BREAKDOWN;
@@ -218,18 +227,14 @@ static int solve_linear(bo_sim* s, double tol, int maxit, int* its) {
         *its = 0;
         return LS_BREAKDOWN;
     }
-    if (s->precond == BO_PRECOND_CPR) {   // a singular pivot of the coarsest pressure operator
-        int bad = 0;
-        BO_CUDA(cudaMemcpy(&bad, cpr_status_ptr(s), sizeof(int), cudaMemcpyDeviceToHost));
-        if (bad) {
-            *its = 0;
-            return LS_BREAKDOWN;
-        }
+    if (s->h_flags->cpr_singular) {   // a singular pivot of the coarsest pressure operator
+        *its = 0;
+        return LS_BREAKDOWN;
     }
     s->factored = true;
     s->last_fallback = 0;
     int st = run_bicgstab(s, tol, maxit, its, true);
-    check_timeout(s);
+    check_timeout_read(s);
     if (st != LS_OK && s->ml_on) {
         // the learned stage failed on this system: repeat with plain ILU(0)
         s->ml_fallbacks += 1;
@@ -328,7 +333,6 @@ static int newton(bo_sim* s, double dt, const bo_newton_opts& o, int* nits, int*
         int li = 0;
         t0 = clk::now();
         int st = solve_linear(s, o.tol_lin, o.max_lin, &li);
-        sync(s);
         rep->ms_solve += ms_since(t0);
         *lits += li;
         if (st != LS_OK) {  // breakdown or missed tolerance fails the Newton solve
@@ -406,6 +410,7 @@ bo_status bo_create_grid(int nx, int ny, int nz, const double* dx, const double*
             BO_CUDA(cudaMemset(s->d_ns, 0, sizeof(NewtonStatus)));
             BO_CUDA(cudaMallocHost(reinterpret_cast<void**>(&s->h_ns), sizeof(NewtonStatus)));
             BO_CUDA(cudaMallocHost(reinterpret_cast<void**>(&s->h_ks), sizeof(KrylovScalars)));
+            BO_CUDA(cudaMallocHost(reinterpret_cast<void**>(&s->h_flags), sizeof(SolveFlags)));
             setup_sweeps(s);
         } catch (...) {
             free_all(s);

@@ -494,6 +494,7 @@ int run_block_bicgstab(bo_sim* s, double tol, int maxit, int max_restarts, int* 
     timer_end(s, t);
     BO_CUDA(cudaMemcpyAsync(s->h_ks, s->d_ks, sizeof(KrylovScalars), cudaMemcpyDeviceToHost,
                             s->stream));
+    read_flags_async(s);
     BO_CUDA(cudaStreamSynchronize(s->stream));
     timers_flush(s);
     const KrylovScalars& k = *s->h_ks;

@@ -87,6 +87,11 @@ struct KrylovScalars {
     double true_nr;                 // ||b - Op x||_2 at the last check
     double stop;                    // the recurrence stops at ||r|| <= stop
     double inner;                   // per-cycle relative target (0: tol alone)
+    int loops;                      // turns of the iteration loop (launch accounting)
+};
+// What a factorisation and a solve leave for the host, read with one wait.
+struct SolveFlags {
+    int sweep_timeout, cpr_singular;
 };
 enum { KS_RUN = 0, KS_HALF = 1, KS_DONE = 2 };
 enum { LS_OK = 0, LS_NOT_CONVERGED = 1, LS_BREAKDOWN = 2 };
@@ -215,6 +220,7 @@ struct bo_sim {
     bo::NewtonStatus* d_ns = nullptr;
     bo::NewtonStatus* h_ns = nullptr;   // pinned
     bo::KrylovScalars* h_ks = nullptr;  // pinned
+    bo::SolveFlags* h_flags = nullptr;  // pinned
 
     // learned preconditioner stage (learned.cu)
     float* d_ml_theta = nullptr;   // FP32 parameters (BO_LEARN_NPARAM)
@@ -258,6 +264,8 @@ struct bo_sim {
 
     // CUDA graphs of one BiCGStab iteration block and of the factorisation
     cudaGraphExec_t g_iter = nullptr;
+    cudaGraphExec_t g_loop = nullptr;   // iterations in a device-side loop until the recurrence stops
+    int loop_kernels = 0;               // kernels of a turn
     cudaGraphExec_t g_factor = nullptr;
     cudaGraphExec_t g_iter_timed = nullptr;
     int iters_per_graph = 4;
@@ -295,7 +303,7 @@ void launch_well_init_bhp(bo_sim* s);
 void launch_restore(bo_sim* s);
 
 void setup_sweeps(bo_sim* s);
-int sweep_timeout(bo_sim* s);
+void read_flags_async(bo_sim* s);   // h_flags, valid after the next wait for the stream
 void setup_sweeps64(bo_sim* s);                  // FP64 sweep plan for the current boxes
 void free_sweeps64(bo_sim* s);
 void reset_tickets(bo_sim* s);                   // after a change of the sweeps' grid

@@ -144,11 +144,13 @@ void enqueue_bwd(bo_sim* s, cudaStream_t st, double* z, const KrylovScalars* ks)
     enqueue_bwd64(s, st, z, ks);
 }
 
-int sweep_timeout(bo_sim* s) {
-    int v = 0;
-    BO_CUDA(cudaMemcpyAsync(&v, s->d_sweep_sync + 2, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-    BO_CUDA(cudaStreamSynchronize(s->stream));
-    return v;
+void read_flags_async(bo_sim* s) {
+    BO_CUDA(cudaMemcpyAsync(&s->h_flags->sweep_timeout, s->d_sweep_sync + 2, sizeof(int),
+                            cudaMemcpyDeviceToHost, s->stream));
+    s->h_flags->cpr_singular = 0;
+    if (s->precond == BO_PRECOND_CPR)
+        BO_CUDA(cudaMemcpyAsync(&s->h_flags->cpr_singular, cpr_status_ptr(s), sizeof(int),
+                                cudaMemcpyDeviceToHost, s->stream));
 }
 
 // Runs one bounded face wait that can only time out; returns the wait time.

@@ -16,10 +16,11 @@
 // Cells with equal i+j+k (a wavefront level) are independent in both
 // recurrences; levels run in order.
 //
-// BiCGStab (van der Vorst), right preconditioned, all scalars on the device:
-// every kernel reads the recurrence state and returns at once when the solve
-// has finished, so a fixed CUDA graph of several iterations can be replayed
-// until the host sees the finished flag.  Reductions are deterministic:
+// BiCGStab (van der Vorst), right preconditioned, all scalars on the device: the
+// iterations run in a device-side loop of a CUDA graph until the recurrence stops.
+// Every kernel reads the recurrence state and returns at once when the solve has
+// finished, so a fixed graph of several iterations can also be replayed until the
+// host sees the finished flag (timed runs, FP32 sweeps, the learned stage).  Reductions are deterministic:
 // per-block partials in a fixed grid, summed in a fixed order.
 #include <algorithm>
 #include <cmath>
@@ -305,6 +306,7 @@ __global__ void k_s_setup(KrylovScalars* ks, const double* __restrict__ part, in
     ks->half_exit = 0;
     ks->restarts = 0;
     ks->true_nr = ks->nr0;
+    ks->loops = 0;
     ks->inner = inner;
     ks->stop = fmax(tol, inner) * ks->nr0;
     if (ks->nr0 == 0.0) {
@@ -373,29 +375,37 @@ __global__ void k_s4(KrylovScalars* ks, const double* __restrict__ part, int nb)
     ks->omega = om;
 }
 
-// convergence on ||r||; next rho = (rh, r)
-__global__ void k_s5(KrylovScalars* ks, const double* __restrict__ part, int nb) {
-    int st = ks->state;
-    if (st == KS_DONE) return;
-    if (st == KS_HALF) {
-        if (threadIdx.x == 0) {
-            ks->state = KS_DONE;
-            ks->status = LS_OK;
-        }
-        return;
+// convergence on ||r||; next rho = (rh, r).  In the device-side loop (looped) also
+// whether it takes another turn.
+__global__ void k_s5(KrylovScalars* ks, const double* __restrict__ part, int nb, int looped,
+                     cudaGraphConditionalHandle loop) {
+    const int st = ks->state;
+    double rr = 0.0, rhr = 0.0;
+    if (st == KS_RUN) {
+        rr = sum_partials(part, nb);
+        rhr = sum_partials(part + nb, nb);
     }
-    double rr = sum_partials(part, nb);
-    double rhr = sum_partials(part + nb, nb);
     if (threadIdx.x != 0) return;
-    double nr = sqrt(rr);
-    ks->last_nr = nr;
-    if (nr <= ks->stop) {
+    bool more = false;
+    if (st == KS_HALF) {
         ks->state = KS_DONE;
         ks->status = LS_OK;
-        return;
+    } else if (st == KS_RUN) {
+        const double nr = sqrt(rr);
+        ks->last_nr = nr;
+        if (nr <= ks->stop) {
+            ks->state = KS_DONE;
+            ks->status = LS_OK;
+        } else {
+            ks->rho_old = ks->rho;
+            ks->rho = rhr;
+            more = true;
+        }
     }
-    ks->rho_old = ks->rho;
-    ks->rho = rhr;
+    if (looped) {
+        ks->loops += 1;
+        cudaGraphSetConditional(loop, more ? 1u : 0u);
+    }
 }
 
 // The recurrence's residual decides when to stop, the true residual
@@ -407,6 +417,7 @@ __global__ void k_s5(KrylovScalars* ks, const double* __restrict__ part, int nb)
 // application, which limits how far one BiCGStab cycle can reduce the
 // residual).  With allow == 0 the solve is reported as not converged instead.
 __global__ void k_s_restart(KrylovScalars* ks, const double* __restrict__ part, int nb, int allow) {
+    if (ks->status == LS_BREAKDOWN) return;   // nothing to accept
     double rr = sum_partials(part, nb);
     if (threadIdx.x != 0) return;
     double nr = sqrt(rr);
@@ -501,7 +512,7 @@ void count_launch(bo_sim* s, cudaStream_t st, int k) {
     s->launches += k;
 }
 
-void note_graph(bo_sim* s, cudaGraph_t g, cudaGraphExec_t exec) {
+static int kernel_nodes(cudaGraph_t g) {
     size_t count = 0;
     BO_CUDA(cudaGraphGetNodes(g, nullptr, &count));
     std::vector<cudaGraphNode_t> nodes(count);
@@ -512,7 +523,10 @@ void note_graph(bo_sim* s, cudaGraph_t g, cudaGraphExec_t exec) {
         BO_CUDA(cudaGraphNodeGetType(nd, &t));
         if (t == cudaGraphNodeTypeKernel) kernels += 1;
     }
-    s->graph_kernels.emplace_back(exec, kernels);
+    return kernels;
+}
+void note_graph(bo_sim* s, cudaGraph_t g, cudaGraphExec_t exec) {
+    s->graph_kernels.emplace_back(exec, kernel_nodes(g));
 }
 
 void graph_launch(bo_sim* s, cudaGraphExec_t exec, cudaStream_t st) {
@@ -572,7 +586,8 @@ enum { TI_FWD = 0, TI_BWD = 1, TI_SPMV = 2, TI_BLAS = 3, TI_N = 4 };
 
 // ml: the learned correction follows each preconditioner apply (z += delta);
 // collect: the residual of every iteration is stored as a training sample.
-static void enqueue_iteration(bo_sim* s, cudaStream_t st, cudaEvent_t* ev, bool ml, bool collect) {
+static void enqueue_iteration(bo_sim* s, cudaStream_t st, cudaEvent_t* ev, bool ml, bool collect,
+                              const cudaGraphConditionalHandle* loop = nullptr) {
     const int N = 3 * s->geo.n;
     KrylovScalars* ks = s->d_ks;
     double* part = s->d_part;
@@ -642,7 +657,8 @@ static void enqueue_iteration(bo_sim* s, cudaStream_t st, cudaEvent_t* ev, bool 
     count_launch(s, st);
     rec(17);
     if (collect) enqueue_learn_collect(s, st, s->d_r, ks);
-    k_s5<<<1, 256, 0, st>>>(ks, part, VEC_GRID);
+    k_s5<<<1, 256, 0, st>>>(ks, part, VEC_GRID, loop != nullptr,
+                            loop ? *loop : cudaGraphConditionalHandle{});
     count_launch(s, st);
     BO_LAUNCH_CHECK("bicgstab iteration");
 }
@@ -660,6 +676,38 @@ static cudaGraphExec_t capture(bo_sim* s, int iters, cudaEvent_t* ev, bool ml, b
     cudaGraphExec_t exec;
     BO_CUDA(cudaGraphInstantiate(&exec, graph, 0));
     note_graph(s, graph, exec);
+    BO_CUDA(cudaGraphDestroy(graph));
+    BO_CUDA(cudaStreamDestroy(cs));
+    return exec;
+}
+
+// One iteration as the body of a device-side loop (a conditional node that k_s5
+// sets): the solve ends on the device with the iteration that converges.  A graph of
+// four iterations replayed until the host saw the flag cost a wait for the host
+// every four (15 to 20 us) and, after the last, up to three iterations of kernels
+// that return at once (2 us each, 18 with ILU(0), 45 with CPR).
+static cudaGraphExec_t capture_loop(bo_sim* s) {
+    cudaStream_t cs;
+    BO_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+    cudaGraph_t graph, body;
+    BO_CUDA(cudaGraphCreate(&graph, 0));
+    cudaGraphConditionalHandle h;
+    BO_CUDA(cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault));
+    cudaGraphNodeParams np = {};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = h;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    cudaGraphNode_t node;
+    BO_CUDA(cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np));
+    body = np.conditional.phGraph_out[0];
+    BO_CUDA(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    enqueue_iteration(s, cs, nullptr, false, false, &h);
+    cudaGraph_t captured;
+    BO_CUDA(cudaStreamEndCapture(cs, &captured));
+    s->loop_kernels = kernel_nodes(body);
+    cudaGraphExec_t exec;
+    BO_CUDA(cudaGraphInstantiate(&exec, graph, 0));
     BO_CUDA(cudaGraphDestroy(graph));
     BO_CUDA(cudaStreamDestroy(cs));
     return exec;
@@ -685,7 +733,12 @@ static cudaGraphExec_t capture_factor(bo_sim* s) {
 void build_graphs(bo_sim* s) {
     destroy_graphs(s);
     s->g_factor = capture_factor(s);
-    s->g_iter = capture(s, s->iters_per_graph, nullptr, false, learn_collecting(s));
+    // the FP32 sweeps' cooperative launches and the collection of residuals stay
+    // with the replayed graph
+    if (s->mixed || learn_collecting(s))
+        s->g_iter = capture(s, s->iters_per_graph, nullptr, false, learn_collecting(s));
+    else
+        s->g_loop = capture_loop(s);
     if (s->ml_on) s->g_iter_ml = capture(s, s->iters_per_graph, nullptr, true, learn_collecting(s));
     if (s->mixed) {   // FP64 sweeps for a solve the FP32 sweeps fail
         s->mixed = false;
@@ -701,11 +754,12 @@ void build_graphs(bo_sim* s) {
 
 void destroy_graphs(bo_sim* s) {
     if (s->g_iter) cudaGraphExecDestroy(s->g_iter);
+    if (s->g_loop) cudaGraphExecDestroy(s->g_loop);
     if (s->g_factor) cudaGraphExecDestroy(s->g_factor);
     if (s->g_iter_timed) cudaGraphExecDestroy(s->g_iter_timed);
     if (s->g_iter_ml) cudaGraphExecDestroy(s->g_iter_ml);
     if (s->g_iter64) cudaGraphExecDestroy(s->g_iter64);
-    s->g_iter = s->g_factor = s->g_iter_timed = s->g_iter_ml = s->g_iter64 = nullptr;
+    s->g_loop = s->g_iter = s->g_factor = s->g_iter_timed = s->g_iter_ml = s->g_iter64 = nullptr;
     for (cudaEvent_t e : s->iter_events) cudaEventDestroy(e);
     s->iter_events.clear();
     s->graph_kernels.clear();
@@ -792,6 +846,7 @@ static void replay_iterations(bo_sim* s, cudaGraphExec_t g, bool timed, int* pre
     for (int guard = 0; guard < left + 2; guard += s->iters_per_graph) {
         graph_launch(s, g, st);
         BO_CUDA(cudaMemcpyAsync(s->h_ks, s->d_ks, sizeof(KrylovScalars), cudaMemcpyDeviceToHost, st));
+        read_flags_async(s);
         BO_CUDA(cudaStreamSynchronize(st));
         const KrylovScalars& k = *s->h_ks;
         if (timed) {
@@ -865,11 +920,17 @@ int run_bicgstab(bo_sim* s, double tol, int maxit, int* its, bool use_ml, bool f
     cudaGraphExec_t g = timed ? s->g_iter_timed
                         : (s->mixed && !fp32) ? s->g_iter64
                         : (ml ? s->g_iter_ml : s->g_iter);
+    const bool loop = !timed && !ml && s->g_loop;   // (never with the FP32 sweeps)
+    int loops = 0;
     const int t_check = timer_id(s, "true_residual");
     int prev_it = 0;
     for (int round = 0;; ++round) {
-        replay_iterations(s, g, timed, &prev_it);
-        if (s->h_ks->state != KS_DONE || s->h_ks->status == LS_BREAKDOWN) break;
+        if (loop) {
+            graph_launch(s, s->g_loop, st);
+        } else {
+            replay_iterations(s, g, timed, &prev_it);
+            if (s->h_ks->state != KS_DONE || s->h_ks->status == LS_BREAKDOWN) break;
+        }
         // FP64 true residual r = b - Op x; accept, restart from it, or give up
         timer_begin(s, t_check);
         enqueue_op<3>(s, st, s->d_xs, s->d_r, s->d_b, nullptr);
@@ -881,7 +942,12 @@ int run_bicgstab(bo_sim* s, double tol, int maxit, int* its, bool use_ml, bool f
         timer_end(s, t_check);
         BO_LAUNCH_CHECK("true residual");
         BO_CUDA(cudaMemcpyAsync(s->h_ks, s->d_ks, sizeof(KrylovScalars), cudaMemcpyDeviceToHost, st));
+        read_flags_async(s);
         BO_CUDA(cudaStreamSynchronize(st));
+        if (loop) {
+            s->launches += (long long)s->loop_kernels * (s->h_ks->loops - loops);
+            loops = s->h_ks->loops;
+        }
         if (s->h_ks->state != KS_RUN) break;
     }
     timers_flush(s);
