@@ -25,8 +25,10 @@
 //     level; a level of a tile on its own takes 600 cycles, 304 ns.
 //   * The factors are stored lane by lane, a level's 3 KB in one piece: a copy
 //     warp brings them and the right-hand side into a ring in shared memory with
-//     two bulk copies a level, RING levels ahead (cp.async by the compute warps
-//     instead: 343 ns a level; plain loads six levels ahead: 400 ns).
+//     16-byte asynchronous copies, up to RING levels ahead, and announces the
+//     levels that are in (304 ns a level; the copies issued by the compute warps:
+//     343, loads by the face warps through registers: 327, plain loads by the
+//     compute warps six levels ahead: 400).
 //   * Values of the neighbouring tiles come through write-once slots in global
 //     memory that hold a NaN sentinel until written.  Four face warps poll them,
 //     each every fourth level, write them to a ring in shared memory and arrive
@@ -37,8 +39,8 @@
 //     level at which a tile can start).  A tile waits only for tiles with smaller
 //     tickets, which CTAs already running hold, so every wait ends whatever else
 //     shares the GPU and no launch has to be resident as a whole.
-// Measured, a sweep: 60x220x85 262 us (405 before, with one warp per row of an
-// 8 x 4 tile and a handoff per level), 33x27x9 30 us (52.6 before).
+// Measured, a sweep: 60x220x85 267 us (405 before, with one warp per row of an
+// 8 x 4 tile and a handoff per level), 33x27x9 31 us (52.6 before).
 // Waits are bounded; one that runs out sets the error flag and the sweep ends
 // with zeros for the missing values.
 #include <algorithm>
@@ -52,36 +54,11 @@ namespace bo {
 constexpr int SWEEP_THREADS = 32 * (TSJ + FACE_WARPS + 1);   // compute, face and copy warps
 constexpr int SLOT = 3 * LINES;           // doubles of one level in shared memory
 constexpr int STAGE = 96 * TSJ + SLOT;    // doubles of a level: factors, right-hand side
+constexpr int STAGE_LOADS = 96 * TSJ / 64 + 1;   // 16-byte loads of a lane for a level
+static_assert(96 * TSJ % 64 == 0 && SLOT % 2 == 0 && SLOT / 2 <= 32, "a level in whole loads");
 constexpr int FACE_LANES = 3 * (TSK + TSJ);   // face values of one level: j-face, k-face
 static_assert(TSJ + TSK <= LINES && FACE_LANES <= FACE_W, "a level's face values fit a slot");
 
-// mbarriers of the stages and the copies that complete them
-__device__ __forceinline__ void mb_init(unsigned long long* bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sa(bar)) : "memory");
-}
-__device__ __forceinline__ void mb_expect(unsigned long long* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mb_try(unsigned long long* bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(sa(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// global -> shared (16-byte aligned addresses, a multiple of 16 bytes)
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes,
-                                         unsigned long long* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-            "r"(sa(dst)),
-        "l"(src), "r"(bytes), "r"(sa(bar))
-        : "memory");
-}
 // ---------------------------------------------------------------------------
 // q = D^-1 r in the forward sweep's order: its right-hand side, formed by all
 // SMs before the wavefront (9 products a cell, bound by bytes: 72 + 24 in, 24
@@ -106,6 +83,10 @@ k_sweep_rhs(int n, int nx, const unsigned* __restrict__ lb, const double* __rest
     }
 }
 
+__device__ __forceinline__ void copy16(unsigned dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // a8: one sweep.  Compute warp w owns the lines jj = w, lane 9 kk + 3 row + d
 // the chain of row `row` towards neighbour d (0: i-1, 1: j-1, 2: k-1).
@@ -122,20 +103,16 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
     constexpr int PLANE = 0, HALO = 2 * SLOT, ZERO = HALO + RING * SLOT;
     __shared__ double ex[ZERO + SLOT];
     __shared__ __align__(16) double ring[RING][STAGE];   // a level's factors and right-hand side
-    __shared__ unsigned long long bar[RING];
     __shared__ unsigned s_rank;
+    __shared__ int s_copied;                  // levels whose entries have come to the ring
     __shared__ int s_done, s_begun;           // levels begun by the compute warps; level 0 is in
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int NL = a.NL, nx = a.g.nx, n = a.g.n;
 
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < RING; ++q) mb_init(&bar[q]);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    for (int turn = 0;; ++turn) {   // tiles this CTA has done
+    for (;;) {
         if (threadIdx.x == 0) {
             s_rank = draw_tile(a);
-            s_done = s_begun = 0;
+            s_done = s_begun = s_copied = 0;
         }
         for (int q = threadIdx.x; q < 2 * SLOT; q += SWEEP_THREADS) ex[PLANE + q] = 0.0;
         for (int q = threadIdx.x; q < SLOT; q += SWEEP_THREADS) ex[ZERO + q] = 0.0;
@@ -143,29 +120,31 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
         const unsigned rank = s_rank;
         if (rank >= (unsigned)a.T) return;
         const SweepTile t = a.tiles[rank];
-        // parity of level l's mbarrier phase: the uses of its place so far
-        auto parity = [&](int l) {
-            const int uses = (NL - (l & (RING - 1)) + RING - 1) / RING;
-            return (unsigned)(turn * uses + l / RING) & 1u;
-        };
-
         if (warp == TSJ + FACE_WARPS) {
             // ---- copy warp: a level's factors and right-hand side into its place,
             // once the level that held it before has begun (its entries are read
-            // one level earlier) ------------------------------------------------
-            if (lane == 0) {
-                const double* Sp = S + (size_t)rank * NL * (TSJ * 96);
-                const double* Qp = Q + (size_t)rank * NL * SLOT;
-                for (int l = 0; l < NL; ++l) {
+            // one level earlier); levels under way are waited for when no place is
+            // free, and announced ------------------------------------------------
+            const char* Sp = reinterpret_cast<const char*>(S + (size_t)rank * NL * (TSJ * 96)) + 16 * lane;
+            const char* Qp = reinterpret_cast<const char*>(Q + (size_t)rank * NL * SLOT) + 16 * lane;
+            auto begun = [&] { return __shfl_sync(FULL, ld_level(&s_done), 0); };   // as one warp
+            int known = 0, told = 0;   // levels seen begun, levels announced
+            for (int l = 0;; ++l) {
+                if (l == NL || (known + RING <= l && (known = begun()) + RING <= l)) {
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncwarp();
+                    if (told != l && lane == 0) st_level(&s_copied, l);
+                    told = l;
+                    if (l == NL) break;
                     int q = 0;
-                    while (ld_level(&s_done) + RING < l + 1 && ++q < WAIT_LIMIT) __nanosleep(20);
-                    if (q >= WAIT_LIMIT) atomicExch(a.err, 1);
-                    unsigned long long* b = &bar[l & (RING - 1)];
-                    double* dst = ring[l & (RING - 1)];
-                    mb_expect(b, STAGE * 8);
-                    bulk_g2s(dst, Sp + (size_t)l * (TSJ * 96), TSJ * 96 * 8, b);
-                    bulk_g2s(dst + TSJ * 96, Qp + (size_t)l * SLOT, SLOT * 8, b);
+                    while ((known = begun()) + RING <= l && ++q < WAIT_LIMIT) __nanosleep(20);
+                    if (q >= WAIT_LIMIT && lane == 0) atomicExch(a.err, 1);
                 }
+                const unsigned dst = sa(ring[l & (RING - 1)]) + 16 * lane;
+                const char* f = Sp + (size_t)l * (TSJ * 96 * 8);
+#pragma unroll
+                for (int u = 0; u < STAGE_LOADS - 1; ++u) copy16(dst + 512 * u, f + 512 * u);
+                if (lane < SLOT / 2) copy16(dst + TSJ * 96 * 8, Qp + (size_t)l * (SLOT * 8));
             }
         } else if (warp >= TSJ) {
             // ---- face warps: levels warp - TSJ, + FACE_WARPS, ... ------------
@@ -189,13 +168,10 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
                 poll_faces(at, need, v, abort, lane, a.err);
                 if (lane < FACE_LANES) ex[to + ((l + 1) & (RING - 1)) * SLOT] = v[0];
                 if (l == 0 && lane == 0) st_level(&s_begun, 1);
-                // the next level's factors (the first one's too) are in
-                for (int m = l == 0 ? 0 : l + 1; m <= l + 1 && m < NL; ++m)
-                    for (q = 0; !__all_sync(FULL, mb_try(&bar[m & (RING - 1)], parity(m))); ++q)
-                        if (q >= WAIT_LIMIT / 16) {
-                            if (lane == 0) atomicExch(a.err, 1);
-                            break;
-                        }
+                // the next level's entries (the first one's too) are in
+                const int last = min(l + 1, NL - 1);
+                for (q = 0; ld_level(&s_copied) <= last && ++q < WAIT_LIMIT;) {}
+                if (q >= WAIT_LIMIT && lane == 0) atomicExch(a.err, 1);
                 __syncwarp();
                 level_arrive(l & (RING - 1));
                 if (need[0]) st_relaxed(at[0], sent);
