@@ -505,7 +505,7 @@ bo_status bo_set_properties(bo_sim* s, const double* perm, const double* poro,
             BO_CUDA(cudaMemset(s->d_wC, 0, sizeof(double) * 3 * s->ncon));
         }
         // reduction scratch: props 1/b partials + norm partials, or Krylov partials + well scalars
-        size_t npart = std::max<size_t>(3 * (size_t)props_blocks(s) + 7 * 1024,
+        size_t npart = std::max<size_t>(3 * (size_t)props_blocks(s) + 10 * 1024,
                                         8 * (size_t)(152 * 4) + s->nw + 1);
         dalloc(&s->d_part, npart);
         double *d_rw = nullptr, *d_skin = nullptr;

@@ -250,34 +250,41 @@ __global__ void k_begin_cells(int n, DevFluid F, const double* __restrict__ p,
     bkflag[c] = flag[c];
 }
 
-// One thread per well, sequential over connections (a handful of values).
-__global__ void k_begin_wells(int nw, DevFluid F, WellDev* __restrict__ wells,
-                              const int* __restrict__ con_cell, const double* __restrict__ depth,
-                              const double* __restrict__ p, const double* __restrict__ sw,
-                              const double* __restrict__ x, const uint8_t* __restrict__ flag) {
-    int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= nw) return;
-    WellDev& W = wells[w];
+// One warp per well: a lane evaluates a connection, then the sums run over the
+// connections in order on values taken from the lanes.  Bound by the chain of one
+// cell evaluation per 32 connections (a thread per well, one connection after the
+// other: 19 us with one connection, 61 us with 9, 500 us with 85; now 10, 12 and 42 us).
+__global__ void __launch_bounds__(32)
+k_begin_wells(DevFluid F, WellDev* __restrict__ wells, const int* __restrict__ con_cell,
+              const double* __restrict__ depth, const double* __restrict__ p,
+              const double* __restrict__ sw, const double* __restrict__ x,
+              const uint8_t* __restrict__ flag) {
+    WellDev& W = wells[blockIdx.x];
+    const int lane = threadIdx.x, off = W.off, ncon = W.ncon, kind = W.kind, phase = W.phase;
+    double rho_well = 0.0, num = 0.0, den = 0.0;
+    const int used = kind == 0 ? 1 : ncon;   // an injector takes its first connection's fluid
+    for (int q0 = 0; q0 < used; q0 += 32) {
+        const int c = con_cell[off + min(q0 + lane, used - 1)];
+        CellD cd;
+        cell_eval(F, p[c], sw[c], x[c], flag[c], cd);
+        if (kind == 0) {
+            rho_well = phase == W_ ? cd.rho[W_].v : phase == O_ ? cd.rho[O_].v : cd.rho[G_].v;
+        } else {
+            for (int q = 0; q < min(32, used - q0); ++q)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const double lam = __shfl_sync(0xffffffffu, cd.lam[a].v, q);
+                    num += lam * __shfl_sync(0xffffffffu, cd.rho[a].v, q);
+                    den += lam;
+                }
+        }
+    }
+    if (lane != 0) return;
+    if (kind != 0) rho_well = den > 0.0 ? num / den : 0.0;
     W.ctl = W.ctl0;
     if (W.ctl == 1) W.bhp = W.target;
-    int c0 = con_cell[W.off];
-    W.z_datum = depth[c0];
-    CellD cd;
-    if (W.kind == 0) {
-        cell_eval(F, p[c0], sw[c0], x[c0], flag[c0], cd);
-        W.rho_well = cd.rho[W.phase].v;
-    } else {
-        double num = 0.0, den = 0.0;
-        for (int q = 0; q < W.ncon; ++q) {
-            int c = con_cell[W.off + q];
-            cell_eval(F, p[c], sw[c], x[c], flag[c], cd);
-            for (int a = 0; a < 3; ++a) {
-                num += cd.lam[a].v * cd.rho[a].v;
-                den += cd.lam[a].v;
-            }
-        }
-        W.rho_well = den > 0.0 ? num / den : 0.0;
-    }
+    W.z_datum = depth[con_cell[off]];
+    W.rho_well = rho_well;
     W.bhp_bk = W.bhp;
     if (W.full) {   // full standard well: storage at the step start, backup
         W.xs[3] = W.bhp;
@@ -309,7 +316,12 @@ __global__ void k_restore(int n, double* __restrict__ p, double* __restrict__ sw
 // ---------------------------------------------------------------------------
 // a2 + a3: cell quantities and accumulation (one thread per cell).
 // ---------------------------------------------------------------------------
-constexpr int PROPS_BS = 256;
+// About 460 FP64 operations a cell.  64 threads, so that a small model's warps are
+// spread over the SMs: an FP64 instruction takes 64 cycles, and eight warps on one
+// SM wait for each other (154 cycles each).  33x27x9 19 us, 10x10x3 19 us (37
+// and 37 with 256 threads); with many cells it is the pipe either way (60x220x85
+// 1018 us, 1017 before).
+constexpr int PROPS_BS = 64;
 
 __global__ void __launch_bounds__(PROPS_BS)
 k_props(int n, DevFluid F, const double* __restrict__ p, const double* __restrict__ sw,
@@ -697,13 +709,13 @@ __global__ void k_well_init_bhp(DevFluid F, WellDev* __restrict__ wells,
 // ---------------------------------------------------------------------------
 // a6: convergence measures (Section 2.3).
 // ---------------------------------------------------------------------------
-constexpr int NORM_BS = 256;
+// 64 threads, as for k_props; per block: 3 sum R, 3 max |R|/pv, sum pv, 3 sum 1/b
+constexpr int NORM_BS = 64, NORM_Q = 10;
 
 __global__ void __launch_bounds__(NORM_BS)
-k_norm_partials(int n, const double* __restrict__ R, const double* __restrict__ pv,
-                double* __restrict__ part) {
-    // part[block*7 + {0..2 sum R, 3..5 max |R|/pv, 6 sum pv}]
-    double s[3] = {0, 0, 0}, mx[3] = {0, 0, 0}, spv = 0.0;
+k_norm_partials(int n, const double* __restrict__ R, const double* __restrict__ pv, int nb_props,
+                const double* __restrict__ part_binv, double* __restrict__ part) {
+    double s[3] = {0, 0, 0}, mx[3] = {0, 0, 0}, spv = 0.0, binv[3] = {0, 0, 0};
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
         double v = pv[c];
         spv += v;
@@ -714,11 +726,15 @@ k_norm_partials(int n, const double* __restrict__ R, const double* __restrict__ 
             mx[a] = fmax(mx[a], fabs(r) / v);
         }
     }
-    __shared__ double sh[7][NORM_BS / 32];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double vals[7] = {s[0], s[1], s[2], mx[0], mx[1], mx[2], spv};
+    // the blocks of k_props that fall to this block
+    for (int b = blockIdx.x + gridDim.x * threadIdx.x; b < nb_props; b += gridDim.x * NORM_BS)
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
+        for (int a = 0; a < 3; ++a) binv[a] += part_binv[b * 3 + a];
+    __shared__ double sh[NORM_Q][NORM_BS / 32];
+    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double vals[NORM_Q] = {s[0], s[1], s[2], mx[0], mx[1], mx[2], spv, binv[0], binv[1], binv[2]};
+#pragma unroll
+    for (int q = 0; q < NORM_Q; ++q) {
         double v = vals[q];
         for (int o = 16; o > 0; o >>= 1) {
             double w = __shfl_down_sync(0xffffffffu, v, o);
@@ -727,63 +743,64 @@ k_norm_partials(int n, const double* __restrict__ R, const double* __restrict__ 
         if (lane == 0) sh[q][wid] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 7) {
+    if (threadIdx.x < NORM_Q) {
         int q = threadIdx.x;
         double v = sh[q][0];
         for (int w = 1; w < NORM_BS / 32; ++w) v = (q >= 3 && q < 6) ? fmax(v, sh[q][w]) : v + sh[q][w];
-        part[blockIdx.x * 7 + q] = v;
+        part[blockIdx.x * NORM_Q + q] = v;
     }
 }
 
-__global__ void k_norm_final(int n, int nb_norm, const double* __restrict__ part,
-                             int nb_props, const double* __restrict__ part_binv, double dt,
-                             int nw, const WellDev* __restrict__ wells,
-                             NewtonStatus* __restrict__ ns) {
-    // single warp, fixed-order reduction
-    __shared__ double acc[10];
-    if (threadIdx.x < 10) {
-        int q = threadIdx.x;
-        double v = 0.0;
-        if (q < 7) {
-            for (int b = 0; b < nb_norm; ++b) {
-                double w = part[b * 7 + q];
-                v = (q >= 3 && q < 6) ? fmax(v, w) : v + w;
-            }
-        } else {
-            for (int b = 0; b < nb_props; ++b) v += part_binv[b * 3 + (q - 7)];
+// One warp a quantity, a last one for the wells; sums in a fixed order.  A lane
+// adds at most 1024 / 32 partials (one thread a quantity, one chain over all
+// blocks: 12 us on 33x27x9, 360 us on 60x220x85; now 6 and 11 us).
+__global__ void __launch_bounds__(32 * (NORM_Q + 1))
+k_norm_final(int n, int nb, const double* __restrict__ part, double dt, int nw,
+             const WellDev* __restrict__ wells, NewtonStatus* __restrict__ ns) {
+    __shared__ double acc[NORM_Q + 1];
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool top = q >= 3 && q != 6 && (q < 6 || q == NORM_Q);   // a maximum, not a sum
+    double v = 0.0;
+    if (q < NORM_Q) {
+#pragma unroll 4
+        for (int b = lane; b < nb; b += 32) {
+            const double w = part[b * NORM_Q + q];
+            v = top ? fmax(v, w) : v + w;
         }
-        acc[q] = v;
-    }
-    __syncwarp();
-    if (threadIdx.x == 0) {
-        double pvt = acc[6];
-        for (int a = 0; a < 3; ++a) {
-            double bavg = acc[7 + a] / n;
-            ns->norms[a] = dt * bavg * fabs(acc[a]) / pvt;
-            ns->norms[3 + a] = dt * bavg * acc[3 + a];
-        }
-        double wr = 0.0;
-        for (int w = 0; w < nw; ++w) {
+    } else {
+        for (int w = lane; w < nw; w += 32) {
             const WellDev& W = wells[w];
             if (W.full) {
                 // balances relative to the well's rate scale, fixed fractions
                 // absolute, the control relative to its target
                 const double qs = fmax(fabs(W.xs[0]), 1e-12);
                 if (W.kind == 0) {
-                    wr = fmax(wr, fabs(W.Rs[0]) / qs);
-                    wr = fmax(wr, fmax(fabs(W.Rs[1]), fabs(W.Rs[2])));
+                    v = fmax(v, fabs(W.Rs[0]) / qs);
+                    v = fmax(v, fmax(fabs(W.Rs[1]), fabs(W.Rs[2])));
                 } else {
-                    wr = fmax(wr, fmax(fmax(fabs(W.Rs[0]), fabs(W.Rs[1])), fabs(W.Rs[2])) / qs);
+                    v = fmax(v, fmax(fmax(fabs(W.Rs[0]), fabs(W.Rs[1])), fabs(W.Rs[2])) / qs);
                 }
                 const double scale =
                     (W.ctl == 0) ? W.target : fmax(W.ctl0 == 1 ? W.target : W.limit, 1.0);
-                wr = fmax(wr, fabs(W.Rs[3]) / scale);
+                v = fmax(v, fabs(W.Rs[3]) / scale);
             } else if (W.ctl == 0) {
-                wr = fmax(wr, fabs(W.Rw) / fmax(fabs(W.target), 1e-300));
+                v = fmax(v, fabs(W.Rw) / fmax(fabs(W.target), 1e-300));
             }
         }
-        ns->norms[6] = wr;
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double w = __shfl_down_sync(0xffffffffu, v, o);
+        v = top ? fmax(v, w) : v + w;
+    }
+    if (lane == 0) acc[q] = v;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        const double bavg = acc[7 + a] / n;
+        ns->norms[a] = dt * bavg * fabs(acc[a]) / acc[6];
+        ns->norms[3 + a] = dt * bavg * acc[3 + a];
+    }
+    if (threadIdx.x == 3) ns->norms[6] = acc[NORM_Q];
 }
 
 // ---------------------------------------------------------------------------
@@ -907,7 +924,7 @@ void launch_hydrostatic(bo_sim* s, double p_top, double sw, double rgo) {
 
 void launch_begin_step(bo_sim* s) {
     int n = s->geo.n;
-    k_begin_cells<<<blocks_for(n, 256), 256, 0, s->stream>>>(n, s->fluid, s->d_p, s->d_sw,
+    k_begin_cells<<<blocks_for(n, PROPS_BS), PROPS_BS, 0, s->stream>>>(n, s->fluid, s->d_p, s->d_sw,
                                                             s->d_x, s->d_flag, s->d_A0,
                                                             s->d_bk, s->d_bkflag);
     count_launch(s, s->stream);
@@ -917,9 +934,8 @@ void launch_begin_step(bo_sim* s) {
 
 void launch_begin_wells(bo_sim* s) {
     if (s->nw == 0) return;
-    k_begin_wells<<<blocks_for(s->nw, 32), 32, 0, s->stream>>>(
-        s->nw, s->fluid, s->d_wells, s->d_con_cell, s->d_depth, s->d_p, s->d_sw, s->d_x,
-        s->d_flag);
+    k_begin_wells<<<s->nw, 32, 0, s->stream>>>(s->fluid, s->d_wells, s->d_con_cell, s->d_depth,
+                                               s->d_p, s->d_sw, s->d_x, s->d_flag);
     count_launch(s, s->stream);
     BO_LAUNCH_CHECK("k_begin_wells");
 }
@@ -993,11 +1009,11 @@ void launch_norms(bo_sim* s, double dt) {
     int nb = norm_blocks(s);
     int npb = props_blocks(s);
     double* part_norm = s->d_part + 3 * (size_t)npb;
-    k_norm_partials<<<nb, NORM_BS, 0, s->stream>>>(n, s->d_R, s->d_pv, part_norm);
+    k_norm_partials<<<nb, NORM_BS, 0, s->stream>>>(n, s->d_R, s->d_pv, npb, s->d_part, part_norm);
     count_launch(s, s->stream);
     BO_LAUNCH_CHECK("k_norm_partials");
-    k_norm_final<<<1, 32, 0, s->stream>>>(n, nb, part_norm, npb, s->d_part, dt, s->nw,
-                                          s->d_wells, s->d_ns);
+    k_norm_final<<<1, 32 * (NORM_Q + 1), 0, s->stream>>>(n, nb, part_norm, dt, s->nw, s->d_wells,
+                                                        s->d_ns);
     count_launch(s, s->stream);
     BO_LAUNCH_CHECK("k_norm_final");
 }
