@@ -379,7 +379,13 @@ k_props(int n, DevFluid F, const double* __restrict__ p, const double* __restric
 }
 
 // ---------------------------------------------------------------------------
-// a4: face fluxes with upwinding (one thread per cell, six faces).
+// a4: face fluxes with upwinding.  k_faces evaluates every face once and writes
+// the two off-diagonal blocks; k_flux_sums adds them up for each cell.
+//
+// Bound by FP64 operations, about 110 a face.  A thread per cell that went over its
+// six faces evaluated each face twice, and on a small model one such chain of 800
+// operations was the whole time: 35 us on 33x27x9, 1728 us on 60x220x85.  Now
+// 9 + 9 us and 759 + 162 us.
 // ---------------------------------------------------------------------------
 struct FaceSide {
     double rho[3][4];   // value + 3 derivatives
@@ -410,113 +416,115 @@ __device__ __forceinline__ void load_side(const double* __restrict__ props,
 __device__ __forceinline__ void face_flux(const FaceSide& L, const FaceSide& H, double T,
                                           double g, double u[3], double dl[3][3],
                                           double dh[3][3]) {
-    double dz = L.z - H.z;
+    const double dz = L.z - H.z, dp = L.p - H.p;
+    const double hg = 0.5 * g;   // a factor 1/2 rounds nothing
     double phv[3], phl[3][3], phh[3][3];
     bool upl[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        double rij = 0.5 * (L.rho[a][0] + H.rho[a][0]);
-        double grav = g * rij;
-        phv[a] = (L.p - H.p) - grav * dz;
+        phv[a] = dp - (hg * (L.rho[a][0] + H.rho[a][0])) * dz;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            phl[a][k] = (k == 0 ? 1.0 : 0.0) - (g * (0.5 * L.rho[a][1 + k])) * dz;
-            phh[a][k] = (k == 0 ? -1.0 : 0.0) - (g * (0.5 * H.rho[a][1 + k])) * dz;
+            phl[a][k] = (k == 0 ? 1.0 : 0.0) - (hg * L.rho[a][1 + k]) * dz;
+            phh[a][k] = (k == 0 ? -1.0 : 0.0) - (hg * H.rho[a][1 + k]) * dz;
         }
         upl[a] = phv[a] >= 0.0;
-        const double* m = upl[a] ? L.mob[a] : H.mob[a];
-        double mt = m[0] * T;
+        const double mt = (upl[a] ? L.mob[a][0] : H.mob[a][0]) * T;
         u[a] = mt * phv[a];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            double up = (m[1 + k] * T) * phv[a];
+            const double up = ((upl[a] ? L.mob[a][1 + k] : H.mob[a][1 + k]) * T) * phv[a];
             dl[a][k] = mt * phl[a][k] + (upl[a] ? up : 0.0);
             dh[a][k] = mt * phh[a][k] + (upl[a] ? 0.0 : up);
         }
     }
     // dissolved gas moves with the oil phase
-    const double* rm = upl[O_] ? L.rmob : H.rmob;
-    double rt = rm[0] * T;
+    const double rt = (upl[O_] ? L.rmob[0] : H.rmob[0]) * T;
     u[G_] = u[G_] + rt * phv[O_];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        double up = (rm[1 + k] * T) * phv[O_];
+        const double up = ((upl[O_] ? L.rmob[1 + k] : H.rmob[1 + k]) * T) * phv[O_];
         dl[G_][k] = dl[G_][k] + (rt * phl[O_][k] + (upl[O_] ? up : 0.0));
         dh[G_][k] = dh[G_][k] + (rt * phh[O_][k] + (upl[O_] ? 0.0 : up));
     }
 }
 
-constexpr int FLUX_BS = 128;
+// The faces' fluxes at [axis n + lower cell]: vectors of the Krylov solver, which
+// sets them anew at the start of a solve.
+struct FaceFlux {
+    double* u[3];
+};
 
-__global__ void __launch_bounds__(FLUX_BS)
-k_flux(Geom g, double grav, const double* __restrict__ props, const double* __restrict__ p,
-       const double* __restrict__ depth, const double* __restrict__ T,
-       double* __restrict__ R, double* __restrict__ A) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    int n = g.n;
+constexpr int FACE_BS = 64, FLUX_BS = 64;
+
+// One thread per cell and axis (blockIdx.y): the face towards the next cell.
+__global__ void __launch_bounds__(FACE_BS)
+k_faces(Geom g, double grav, const double* __restrict__ props, const double* __restrict__ p,
+        const double* __restrict__ depth, const double* __restrict__ T, double* __restrict__ A,
+        FaceFlux f) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, n = g.n, axis = blockIdx.y;
     if (c >= n) return;
-    int i = c % g.nx, j = (c / g.nx) % g.ny, k = c / (g.nx * g.ny);
-    int plane = g.nx * g.ny;
-    FaceSide me, nb;
-    load_side(props, p, depth, n, c, me);
-    double r[3], jd[9];
+    const int jk = c / g.nx;
+    const int at = axis == 0 ? c - jk * g.nx : axis == 1 ? jk % g.ny : jk / g.ny;
+    const int len = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz;
+    const int step = axis == 0 ? 1 : axis == 1 ? g.nx : g.nx * g.ny;
+    double* const minus = A + (size_t)((NB_MX + 2 * axis) * 9) * n + c;   // towards the cell before
+    double* const plus = minus + 9 * (size_t)n;
+    if (at == 0)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) r[a] = R[a * n + c];
+        for (int e = 0; e < 9; ++e) minus[(size_t)e * n] = 0.0;
+    if (at + 1 == len) {
 #pragma unroll
-    for (int e = 0; e < 9; ++e) jd[e] = A[e * n + c];
-    // directions in accumulation order: -z, -y, -x, +x, +y, +z
-    const int dirs[6] = {NB_MZ, NB_MY, NB_MX, NB_PX, NB_PY, NB_PZ};
-#pragma unroll 1
-    for (int q = 0; q < 6; ++q) {
-        int b = dirs[q];
-        int other;
-        bool exists;
-        double Tf;
-        switch (b) {
-            case NB_MZ: exists = k > 0; other = c - plane; break;
-            case NB_MY: exists = j > 0; other = c - g.nx; break;
-            case NB_MX: exists = i > 0; other = c - 1; break;
-            case NB_PX: exists = i + 1 < g.nx; other = c + 1; break;
-            case NB_PY: exists = j + 1 < g.ny; other = c + g.nx; break;
-            default:    exists = k + 1 < g.nz; other = c + plane; break;
-        }
-        double* blk = A + (size_t)(b * 9) * n + c;
-        if (!exists) {
+        for (int e = 0; e < 9; ++e) plus[(size_t)e * n] = 0.0;
+        return;
+    }
+    FaceSide lo, hi;
+    load_side(props, p, depth, n, c, lo);
+    load_side(props, p, depth, n, c + step, hi);
+    double u[3], dl[3][3], dh[3][3];
+    face_flux(lo, hi, T[axis * n + c], grav, u, dl, dh);
 #pragma unroll
-            for (int e = 0; e < 9; ++e) blk[(size_t)e * n] = 0.0;
-            continue;
-        }
-        int axis = (b - 1) >> 1;               // 0 x, 1 y, 2 z
-        bool minus = (b & 1) == 1;             // -x, -y, -z
-        int lo = minus ? other : c;
-        Tf = T[axis * n + lo];
-        load_side(props, p, depth, n, other, nb);
-        double u[3], dl[3][3], dh[3][3];
-        if (minus) face_flux(nb, me, Tf, grav, u, dl, dh);
-        else       face_flux(me, nb, Tf, grav, u, dl, dh);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!minus) {          // this cell is the lower one: +u, own derivs dl
-                r[a] += u[a];
-#pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    jd[3 * a + s] += dl[a][s];
-                    blk[(size_t)(3 * a + s) * n] = dh[a][s];
-                }
-            } else {               // this cell is the higher one: -u, own derivs dh
-                r[a] -= u[a];
-#pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    jd[3 * a + s] -= dh[a][s];
-                    blk[(size_t)(3 * a + s) * n] = -dl[a][s];
-                }
-            }
-        }
+    for (int e = 0; e < 9; ++e) {
+        plus[(size_t)e * n] = dh[e / 3][e % 3];
+        minus[(size_t)e * n + step] = -dl[e / 3][e % 3];
     }
 #pragma unroll
-    for (int a = 0; a < 3; ++a) R[a * n + c] = r[a];
+    for (int a = 0; a < 3; ++a) f.u[a][(size_t)axis * n + c] = u[a];
+}
+
+// One thread per cell: residual and diagonal block from the faces.  A face adds
+// +u and its own derivatives to the lower cell, -u to the higher one.
+__global__ void __launch_bounds__(FLUX_BS)
+k_flux_sums(Geom g, FaceFlux f, double* __restrict__ R, double* __restrict__ A) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, n = g.n;
+    if (c >= n) return;
+    const int jk = c / g.nx, i = c - jk * g.nx, k = jk / g.ny, j = jk - k * g.ny;
+    const int plane = g.nx * g.ny;
+    double r[3], jd[9];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) A[e * n + c] = jd[e];
+    for (int a = 0; a < 3; ++a) r[a] = R[(size_t)a * n + c];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) jd[e] = A[(size_t)e * n + c];
+    auto add = [&](int axis, bool minus, int other) {
+        const size_t o = (size_t)axis * n + (minus ? other : c);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) r[a] = minus ? r[a] - f.u[a][o] : r[a] + f.u[a][o];
+        // the derivatives with respect to this cell stand, negated, in the other
+        // cell's block towards it
+        const double* blk = A + (size_t)((NB_MX + 2 * axis + (minus ? 1 : 0)) * 9) * n + other;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) jd[e] -= blk[(size_t)e * n];
+    };
+    if (k > 0) add(2, true, c - plane);
+    if (j > 0) add(1, true, c - g.nx);
+    if (i > 0) add(0, true, c - 1);
+    if (i + 1 < g.nx) add(0, false, c + 1);
+    if (j + 1 < g.ny) add(1, false, c + g.nx);
+    if (k + 1 < g.nz) add(2, false, c + plane);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) R[(size_t)a * n + c] = r[a];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) A[(size_t)e * n + c] = jd[e];
 }
 
 // ---------------------------------------------------------------------------
@@ -968,11 +976,14 @@ void launch_assemble(bo_sim* s, double dt) {
     BO_LAUNCH_CHECK("k_props");
     timer_end(s, tp);
     timer_begin(s, tf);
-    k_flux<<<blocks_for(n, FLUX_BS), FLUX_BS, 0, s->stream>>>(s->geo, s->fluid.g, s->d_props,
-                                                             s->d_p, s->d_depth, s->d_T, s->d_R,
-                                                             s->d_A);
+    const FaceFlux f{{s->d_rh, s->d_pk, s->d_v}};
+    k_faces<<<dim3(blocks_for(n, FACE_BS), 3), FACE_BS, 0, s->stream>>>(
+        s->geo, s->fluid.g, s->d_props, s->d_p, s->d_depth, s->d_T, s->d_A, f);
     count_launch(s, s->stream);
-    BO_LAUNCH_CHECK("k_flux");
+    BO_LAUNCH_CHECK("k_faces");
+    k_flux_sums<<<blocks_for(n, FLUX_BS), FLUX_BS, 0, s->stream>>>(s->geo, f, s->d_R, s->d_A);
+    count_launch(s, s->stream);
+    BO_LAUNCH_CHECK("k_flux_sums");
     timer_end(s, tf);
     BO_CUDA(cudaMemsetAsync(&s->d_ns->dead_wells, 0, sizeof(int), s->stream));
     if (s->well_model == BO_WELL_MODEL_STANDARD) {
