@@ -506,7 +506,7 @@ bo_status bo_set_properties(bo_sim* s, const double* perm, const double* poro,
         }
         // reduction scratch: props 1/b partials + norm partials, or Krylov partials + well scalars
         size_t npart = std::max<size_t>(3 * (size_t)props_blocks(s) + 10 * 1024,
-                                        8 * (size_t)(152 * 4) + s->nw + 1);
+                                        (size_t)KRYLOV_PART + s->nw + 1);
         dalloc(&s->d_part, npart);
         double *d_rw = nullptr, *d_skin = nullptr;
         dalloc(&d_rw, s->nw);

@@ -412,6 +412,7 @@ void timers_flush(bo_sim* s);
 void launch_wi(bo_sim* s, const int* d_con_well, const double* d_rw, const double* d_skin);
 int props_blocks(const bo_sim* s);
 int norm_blocks(const bo_sim* s);
+constexpr int KRYLOV_PART = 8 * 152 * 4;   // doubles of d_part for the Krylov sums; the wells' scalars follow
 
 void residual_norms_noalloc(const double* R, const double* pv, const double* b, int n, double dt,
                             double* out6, cudaStream_t stream);

@@ -31,6 +31,35 @@ namespace bo {
 
 constexpr int VEC_BS = 256;
 constexpr int VEC_GRID = 152 * 4;   // one wave of 4 blocks per SM
+constexpr int SUM_WARPS = VEC_BS / 32;   // warps whose partials make one term of a sum
+
+// Threads of the operator (elements: cells) and the vector kernels (entries).  An
+// FP64 instruction takes 64 cycles, and an SM issues one in 19, so the eight warps
+// of a block wait for each other (154 cycles each) while a small launch leaves other
+// SMs idle.  Up to SMALL_TERMS blocks of 256 elements, blocks have 64 threads and the
+// launch has no idle ones (whose reductions took FP64 cycles all the same).  The same
+// elements fall to the same warps, a small launch leaves the sum over a term's
+// SUM_WARPS warps to the scalar step, and the terms that it leaves out are zeros, so a
+// sum has the same bits either way.  With more terms than the scalar step has threads
+// that step costs what the launch gains.  256 and 64 threads:
+//   operator, 8,019 cells 9.9 and 7.1 us, 51,300 cells 15.7 and 11.6 us
+//   k_xr_update and k_s5, 24,057 entries 5.5 + 6.4 and 2.9 + 6.3 us, 153,900 entries
+//   7.0 + 6.7 and 6.5 + 9.6 us
+constexpr int SUM_BS = 256;   // threads of a scalar step
+constexpr int SMALL_BS = 64, SMALL_TERMS = SUM_BS;
+struct VecShape {
+    int grid, bs;     // of the launch
+    int terms, per;   // of its sums: terms of `per` partials
+    bool small() const { return bs == SMALL_BS; }
+};
+static VecShape vec_shape(int elements) {
+    const int terms = (elements + VEC_BS - 1) / VEC_BS;
+    if (terms > SMALL_TERMS) return {VEC_GRID, VEC_BS, VEC_GRID, 1};
+    return {terms * (VEC_BS / SMALL_BS), SMALL_BS, terms, SUM_WARPS};
+}
+static_assert(SMALL_TERMS <= VEC_GRID, "a small launch visits an element once");
+static_assert(2 * SMALL_TERMS * SUM_WARPS <= KRYLOV_PART && 2 * VEC_GRID <= KRYLOV_PART,
+              "partials of two sums");
 
 __device__ __forceinline__ void cell_ijk(const Geom& g, int c, int& i, int& j, int& k) {
     i = c % g.nx;
@@ -40,6 +69,32 @@ __device__ __forceinline__ void cell_ijk(const Geom& g, int c, int& i, int& j, i
 
 __device__ __forceinline__ bool ks_skip(const KrylovScalars* ks) {
     return ks != nullptr && ks->state != KS_RUN;
+}
+
+// Partials of K sums: with 256 threads one per block, with 64 one per warp.
+template <int BS, int K>
+__device__ __forceinline__ void block_partials(double (&v)[K], double* __restrict__ part) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < K; ++q)
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    if constexpr (BS == SMALL_BS) {
+        const int warps = gridDim.x * (BS / 32), w = blockIdx.x * (BS / 32) + wid;
+#pragma unroll
+        for (int q = 0; q < K; ++q)
+            if (lane == 0) part[q * warps + w] = v[q];
+    } else {
+        __shared__ double sh[K][BS / 32];
+#pragma unroll
+        for (int q = 0; q < K; ++q)
+            if (lane == 0) sh[q][wid] = v[q];
+        __syncthreads();
+        if (threadIdx.x < K) {
+            double x = 0.0;
+            for (int w = 0; w < BS / 32; ++w) x += sh[threadIdx.x][w];
+            part[threadIdx.x * gridDim.x + blockIdx.x] = x;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -71,8 +126,8 @@ __global__ void k_wdot(int n, const WellDev* __restrict__ wells, const int* __re
 
 // mode 0: no dots; 1: part0 = (rh, y); 2: part0 = (y, s), part1 = (y, y);
 // 3: y = o1 - Op x (the true residual of b = o1), part0 = (y, y)
-template <int MODE>
-__global__ void __launch_bounds__(VEC_BS)
+template <int MODE, int BS>
+__global__ void __launch_bounds__(BS)
 k_spmv(Geom g, const double* __restrict__ A, const double* __restrict__ x,
        double* __restrict__ y, const int* __restrict__ cellcon,
        const int* __restrict__ con_well, const double* __restrict__ wC,
@@ -131,47 +186,21 @@ k_spmv(Geom g, const double* __restrict__ A, const double* __restrict__ x,
         }
     }
     if (MODE == 0) return;
-    __shared__ double sh[2][VEC_BS / 32];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-        d0 += __shfl_down_sync(0xffffffffu, d0, o);
-        d1 += __shfl_down_sync(0xffffffffu, d1, o);
-    }
-    if (lane == 0) {
-        sh[0][wid] = d0;
-        sh[1][wid] = d1;
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        double v = 0.0;
-        for (int w = 0; w < VEC_BS / 32; ++w) v += sh[threadIdx.x][w];
-        part[threadIdx.x * gridDim.x + blockIdx.x] = v;
+    double d[2] = {d0, d1};
+    if constexpr (MODE == 2) {
+        block_partials<BS>(d, part);
+    } else {
+        double e[1] = {d0};
+        block_partials<BS>(e, part);
     }
 }
 
 // ---------------------------------------------------------------------------
 // BLAS-1 kernels with fused dot partials (vectors of length N = 3n)
 // ---------------------------------------------------------------------------
-template <int K>
-__device__ __forceinline__ void block_partials(double (&v)[K], double* __restrict__ part) {
-    __shared__ double sh[K][VEC_BS / 32];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-        double x = v[q];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sh[q][wid] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < K) {
-        double x = 0.0;
-        for (int w = 0; w < VEC_BS / 32; ++w) x += sh[threadIdx.x][w];
-        part[threadIdx.x * gridDim.x + blockIdx.x] = x;
-    }
-}
-
 // b = R - sum_w C_w (R_w / D_w); x = 0; r = rh = b; p = v = 0; part0 = (r, r)
-__global__ void __launch_bounds__(VEC_BS)
+template <int BS>
+__global__ void __launch_bounds__(BS)
 k_krylov_init(int N, const double* __restrict__ R, double* __restrict__ b,
               double* __restrict__ x, double* __restrict__ r, double* __restrict__ rh,
               double* __restrict__ p, double* __restrict__ v, double* __restrict__ part) {
@@ -185,7 +214,7 @@ k_krylov_init(int N, const double* __restrict__ R, double* __restrict__ b,
         v[q] = 0.0;
         d[0] += bv * bv;
     }
-    block_partials<1>(d, part);
+    block_partials<BS>(d, part);
     (void)R;
 }
 
@@ -219,7 +248,8 @@ k_p_update(int N, const double* __restrict__ r, double* __restrict__ p,
 }
 
 // s = r - alpha v ; part0 = (s, s)
-__global__ void __launch_bounds__(VEC_BS)
+template <int BS>
+__global__ void __launch_bounds__(BS)
 k_s_update(int N, const double* __restrict__ r, const double* __restrict__ v,
            double* __restrict__ s, double* __restrict__ part,
            const KrylovScalars* __restrict__ ks) {
@@ -231,12 +261,13 @@ k_s_update(int N, const double* __restrict__ r, const double* __restrict__ v,
         s[q] = sv;
         d[0] += sv * sv;
     }
-    block_partials<1>(d, part);
+    block_partials<BS>(d, part);
 }
 
 // RUN:  x += alpha ph + omega sh ; r = s - omega t ; part0 = (r, r), part1 = (rh, r)
 // HALF: x += alpha ph
-__global__ void __launch_bounds__(VEC_BS)
+template <int BS>
+__global__ void __launch_bounds__(BS)
 k_xr_update(int N, double* __restrict__ x, const double* __restrict__ ph,
             const double* __restrict__ sh, const double* __restrict__ s,
             const double* __restrict__ t, double* __restrict__ r,
@@ -258,26 +289,52 @@ k_xr_update(int N, double* __restrict__ x, const double* __restrict__ ph,
         d[0] += rv * rv;
         d[1] += rh[q] * rv;
     }
-    block_partials<2>(d, part);
+    block_partials<BS>(d, part);
 }
 
 // ---------------------------------------------------------------------------
 // Scalar steps of the recurrence (one block; fixed-order sums of partials)
 // ---------------------------------------------------------------------------
-__device__ double sum_partials(const double* __restrict__ part, int nb) {
-    // called by the whole block of 256 threads; returns the sum in thread 0
-    __shared__ double sh[256];
-    double v = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) v += part[b];
-    sh[threadIdx.x] = v;
+// K sums of nb terms in thread 0, by a whole block of 256 threads; a term is the sum
+// of `per` partials, in order.  Two sums go down the tree together.
+template <int K>
+__device__ __forceinline__ void sum_partials(const double* __restrict__ part, int nb, int per,
+                                             double (&r)[K]) {
+    __shared__ double sh[K][SUM_BS];
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < K; ++q) r[q] = 0.0;
+    for (int b = t; b < nb; b += SUM_BS)
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            if (per == 1) {
+                r[q] += part[q * nb + b];
+            } else {
+                const double* w = part + (size_t)(q * nb + b) * SUM_WARPS;
+                double x = 0.0;
+#pragma unroll
+                for (int u = 0; u < SUM_WARPS; ++u) x += w[u];
+                r[q] += x;
+            }
+        }
+#pragma unroll
+    for (int q = 0; q < K; ++q) sh[q][t] = r[q];
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    for (int o = SUM_BS / 2; o >= 32; o >>= 1) {
+        if (t < o)
+#pragma unroll
+            for (int q = 0; q < K; ++q) sh[q][t] = r[q] = r[q] + sh[q][t + o];
         __syncthreads();
     }
-    double r = sh[0];
-    __syncthreads();
-    return r;
+    if (t < 32)
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < K; ++q) r[q] += __shfl_down_sync(0xffffffffu, r[q], o);
+}
+__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int nb, int per) {
+    double r[1];
+    sum_partials(part, nb, per, r);
+    return r[0];
 }
 
 __device__ __forceinline__ void breakdown(KrylovScalars* ks) {
@@ -287,9 +344,9 @@ __device__ __forceinline__ void breakdown(KrylovScalars* ks) {
 }
 
 // setup: nr0 = ||b||, rho = (rh, r) = ||b||^2
-__global__ void k_s_setup(KrylovScalars* ks, const double* __restrict__ part, int nb, double tol,
+__global__ void k_s_setup(KrylovScalars* ks, const double* __restrict__ part, int nb, int per, double tol,
                           int maxit, double inner) {
-    double rr = sum_partials(part, nb);
+    double rr = sum_partials(part, nb, per);
     if (threadIdx.x != 0) return;
     ks->tol = tol;
     ks->maxit = maxit;
@@ -316,8 +373,7 @@ __global__ void k_s_setup(KrylovScalars* ks, const double* __restrict__ part, in
 }
 
 // iteration start: rho (already in ks->rho), beta
-__global__ void k_s1(KrylovScalars* ks) {
-    if (ks->state != KS_RUN) return;
+__device__ __forceinline__ void begin_iteration(KrylovScalars* ks) {
     if (ks->it == ks->maxit) {
         ks->state = KS_DONE;
         ks->status = LS_NOT_CONVERGED;
@@ -331,11 +387,16 @@ __global__ void k_s1(KrylovScalars* ks) {
     }
     ks->beta = (rho / ks->rho_old) * (ks->alpha / ks->omega);
 }
+// before the first iteration; in a replayed graph before every one
+__global__ void k_s1(KrylovScalars* ks) {
+    if (ks->state == KS_RUN) begin_iteration(ks);
+}
 
 // alpha = rho / (rh, v)
-__global__ void k_s2(KrylovScalars* ks, const double* __restrict__ part, int nb) {
+__global__ void __launch_bounds__(SUM_BS)
+k_s2(KrylovScalars* ks, const double* __restrict__ part, int nb, int per) {
     if (ks->state != KS_RUN) return;
-    double rv = sum_partials(part, nb);
+    double rv = sum_partials(part, nb, per);
     if (threadIdx.x != 0) return;
     if (rv == 0.0 || !isfinite(rv)) {
         breakdown(ks);
@@ -345,9 +406,10 @@ __global__ void k_s2(KrylovScalars* ks, const double* __restrict__ part, int nb)
 }
 
 // ||s|| <= tol ||r0||: finish with the half step
-__global__ void k_s3(KrylovScalars* ks, const double* __restrict__ part, int nb) {
+__global__ void __launch_bounds__(SUM_BS)
+k_s3(KrylovScalars* ks, const double* __restrict__ part, int nb, int per) {
     if (ks->state != KS_RUN) return;
-    double ss = sum_partials(part, nb);
+    double ss = sum_partials(part, nb, per);
     if (threadIdx.x != 0) return;
     double ns = sqrt(ss);
     if (ns <= ks->stop) {
@@ -358,10 +420,12 @@ __global__ void k_s3(KrylovScalars* ks, const double* __restrict__ part, int nb)
 }
 
 // omega = (t, s) / (t, t)
-__global__ void k_s4(KrylovScalars* ks, const double* __restrict__ part, int nb) {
+__global__ void __launch_bounds__(SUM_BS)
+k_s4(KrylovScalars* ks, const double* __restrict__ part, int nb, int per) {
     if (ks->state != KS_RUN) return;
-    double ts = sum_partials(part, nb);
-    double tt = sum_partials(part + nb, nb);
+    double sum[2];
+    sum_partials(part, nb, per, sum);
+    const double ts = sum[0], tt = sum[1];
     if (threadIdx.x != 0) return;
     if (tt == 0.0 || !isfinite(tt)) {
         breakdown(ks);
@@ -376,30 +440,29 @@ __global__ void k_s4(KrylovScalars* ks, const double* __restrict__ part, int nb)
 }
 
 // convergence on ||r||; next rho = (rh, r).  In the device-side loop (looped) also
-// whether it takes another turn.
-__global__ void k_s5(KrylovScalars* ks, const double* __restrict__ part, int nb, int looped,
-                     cudaGraphConditionalHandle loop) {
+// the start of the next iteration, if there is one.
+__global__ void __launch_bounds__(SUM_BS)
+k_s5(KrylovScalars* ks, const double* __restrict__ part, int nb, int per, int looped,
+     cudaGraphConditionalHandle loop) {
     const int st = ks->state;
-    double rr = 0.0, rhr = 0.0;
-    if (st == KS_RUN) {
-        rr = sum_partials(part, nb);
-        rhr = sum_partials(part + nb, nb);
-    }
+    double sum[2] = {0.0, 0.0};
+    if (st == KS_RUN) sum_partials(part, nb, per, sum);
     if (threadIdx.x != 0) return;
     bool more = false;
     if (st == KS_HALF) {
         ks->state = KS_DONE;
         ks->status = LS_OK;
     } else if (st == KS_RUN) {
-        const double nr = sqrt(rr);
+        const double nr = sqrt(sum[0]);
         ks->last_nr = nr;
         if (nr <= ks->stop) {
             ks->state = KS_DONE;
             ks->status = LS_OK;
         } else {
             ks->rho_old = ks->rho;
-            ks->rho = rhr;
-            more = true;
+            ks->rho = sum[1];
+            if (looped) begin_iteration(ks);
+            more = ks->state == KS_RUN;
         }
     }
     if (looped) {
@@ -416,9 +479,10 @@ __global__ void k_s5(KrylovScalars* ks, const double* __restrict__ part, int nb,
 // (an FP32 preconditioner is not exactly the same linear map at every
 // application, which limits how far one BiCGStab cycle can reduce the
 // residual).  With allow == 0 the solve is reported as not converged instead.
-__global__ void k_s_restart(KrylovScalars* ks, const double* __restrict__ part, int nb, int allow) {
+__global__ void __launch_bounds__(SUM_BS)
+k_s_restart(KrylovScalars* ks, const double* __restrict__ part, int nb, int per, int allow) {
     if (ks->status == LS_BREAKDOWN) return;   // nothing to accept
-    double rr = sum_partials(part, nb);
+    double rr = sum_partials(part, nb, per);
     if (threadIdx.x != 0) return;
     double nr = sqrt(rr);
     ks->true_nr = nr;
@@ -479,8 +543,6 @@ __global__ void k_well_recover(int n, WellDev* __restrict__ wells,
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-static inline int blocks_for(int n, int bs) { return (n + bs - 1) / bs; }
-
 static int* factor_bad(bo_sim* s) { return reinterpret_cast<int*>(&s->d_ns->pad); }
 
 void enqueue_precond_apply(bo_sim* s, cudaStream_t st, const double* r, double* z,
@@ -493,15 +555,16 @@ void enqueue_precond_apply(bo_sim* s, cudaStream_t st, const double* r, double* 
     enqueue_bwd(s, st, z, ks);
 }
 
-static double* d_sop(bo_sim* s) { return s->d_part + 8 * VEC_GRID; }
+static double* d_sop(bo_sim* s) { return s->d_part + KRYLOV_PART; }
 
 template <int MODE>
 static void enqueue_op(bo_sim* s, cudaStream_t st, const double* x, double* y, const double* o1,
                        const KrylovScalars* ks) {
     enqueue_well_dots(s, st, x, ks);
-    k_spmv<MODE><<<VEC_GRID, VEC_BS, 0, st>>>(s->geo, s->d_A, x, y, s->d_cellcon,
-                                              s->d_cellcon + s->geo.n, s->d_wC, d_sop(s),
-                                              well_corr(s), o1, s->d_part, ks);
+    const VecShape v = vec_shape(s->geo.n);
+    const auto kernel = v.small() ? k_spmv<MODE, SMALL_BS> : k_spmv<MODE, VEC_BS>;
+    kernel<<<v.grid, v.bs, 0, st>>>(s->geo, s->d_A, x, y, s->d_cellcon, s->d_cellcon + s->geo.n,
+                                    s->d_wC, d_sop(s), well_corr(s), o1, s->d_part, ks);
     count_launch(s, st);
     BO_LAUNCH_CHECK("k_spmv");
 }
@@ -598,10 +661,13 @@ static void enqueue_iteration(bo_sim* s, cudaStream_t st, cudaEvent_t* ev, bool 
     };
     // events: 0,1 blas(p); 2,3 fwd1; 4,5 bwd1; 6,7 spmv1; 8,9 blas(s); 10,11 fwd2; 12,13 bwd2;
     //         14,15 spmv2; 16,17 blas(xr)
-    k_s1<<<1, 1, 0, st>>>(ks);
-    count_launch(s, st);
+    const VecShape vc = vec_shape(s->geo.n), vv = vec_shape(N);   // over cells, over entries
+    if (!loop) {   // (k_s5 of the iteration before in the device-side loop)
+        k_s1<<<1, 1, 0, st>>>(ks);
+        count_launch(s, st);
+    }
     rec(0);
-    k_p_update<<<VEC_GRID, VEC_BS, 0, st>>>(N, s->d_r, s->d_pk, s->d_v, ks);
+    k_p_update<<<vv.grid, vv.bs, 0, st>>>(N, s->d_r, s->d_pk, s->d_v, ks);
     count_launch(s, st);
     rec(1);
     // ph = M^-1 p
@@ -623,13 +689,14 @@ static void enqueue_iteration(bo_sim* s, cudaStream_t st, cudaEvent_t* ev, bool 
     rec(6);
     enqueue_op<1>(s, st, s->d_ph, s->d_v, s->d_rh, ks);
     rec(7);
-    k_s2<<<1, 256, 0, st>>>(ks, part, VEC_GRID);
+    k_s2<<<1, SUM_BS, 0, st>>>(ks, part, vc.terms, vc.per);
     count_launch(s, st);
     rec(8);
-    k_s_update<<<VEC_GRID, VEC_BS, 0, st>>>(N, s->d_r, s->d_v, s->d_s, part, ks);
+    (vv.small() ? k_s_update<SMALL_BS> : k_s_update<VEC_BS>)<<<vv.grid, vv.bs, 0, st>>>(
+        N, s->d_r, s->d_v, s->d_s, part, ks);
     count_launch(s, st);
     rec(9);
-    k_s3<<<1, 256, 0, st>>>(ks, part, VEC_GRID);
+    k_s3<<<1, SUM_BS, 0, st>>>(ks, part, vv.terms, vv.per);
     count_launch(s, st);
     rec(10);
     if (s->precond == BO_PRECOND_CPR) {
@@ -649,16 +716,16 @@ static void enqueue_iteration(bo_sim* s, cudaStream_t st, cudaEvent_t* ev, bool 
     rec(14);
     enqueue_op<2>(s, st, s->d_sh, s->d_t, s->d_s, ks);
     rec(15);
-    k_s4<<<1, 256, 0, st>>>(ks, part, VEC_GRID);
+    k_s4<<<1, SUM_BS, 0, st>>>(ks, part, vc.terms, vc.per);
     count_launch(s, st);
     rec(16);
-    k_xr_update<<<VEC_GRID, VEC_BS, 0, st>>>(N, s->d_xs, s->d_ph, s->d_sh, s->d_s, s->d_t,
-                                             s->d_r, s->d_rh, part, ks);
+    (vv.small() ? k_xr_update<SMALL_BS> : k_xr_update<VEC_BS>)<<<vv.grid, vv.bs, 0, st>>>(
+        N, s->d_xs, s->d_ph, s->d_sh, s->d_s, s->d_t, s->d_r, s->d_rh, part, ks);
     count_launch(s, st);
     rec(17);
     if (collect) enqueue_learn_collect(s, st, s->d_r, ks);
-    k_s5<<<1, 256, 0, st>>>(ks, part, VEC_GRID, loop != nullptr,
-                            loop ? *loop : cudaGraphConditionalHandle{});
+    k_s5<<<1, SUM_BS, 0, st>>>(ks, part, vv.terms, vv.per, loop != nullptr,
+                               loop ? *loop : cudaGraphConditionalHandle{});
     count_launch(s, st);
     BO_LAUNCH_CHECK("bicgstab iteration");
 }
@@ -885,7 +952,8 @@ static void replay_iterations(bo_sim* s, cudaGraphExec_t g, bool timed, int* pre
 // Right-hand side of the reduced system into d_b: b = R - sum_w C_w D_w^-1 R_w.
 void enqueue_reduced_rhs(bo_sim* s, cudaStream_t st) {
     const int n = s->geo.n, N = 3 * n;
-    k_rhs_copy<<<VEC_GRID, VEC_BS, 0, st>>>(N, s->d_R, s->d_b);
+    const VecShape vv = vec_shape(N);
+    k_rhs_copy<<<vv.grid, vv.bs, 0, st>>>(N, s->d_R, s->d_b);
     count_launch(s, st);
     if (s->well_model == BO_WELL_MODEL_STANDARD) {
         enqueue_std_wells_rhs(s, st, s->d_b);
@@ -900,14 +968,15 @@ int run_bicgstab(bo_sim* s, double tol, int maxit, int* its, bool use_ml, bool f
     const int N = 3 * s->geo.n;
     cudaStream_t st = s->stream;
     enqueue_reduced_rhs(s, st);
-    k_krylov_init<<<VEC_GRID, VEC_BS, 0, st>>>(N, s->d_R, s->d_b, s->d_xs, s->d_r, s->d_rh,
-                                               s->d_pk, s->d_v, s->d_part);
+    const VecShape vc = vec_shape(s->geo.n), vv = vec_shape(N);
+    (vv.small() ? k_krylov_init<SMALL_BS> : k_krylov_init<VEC_BS>)<<<vv.grid, vv.bs, 0, st>>>(
+        N, s->d_R, s->d_b, s->d_xs, s->d_r, s->d_rh, s->d_pk, s->d_v, s->d_part);
     count_launch(s, st);
     // the learned stage (like the FP32 sweeps) is not the same linear map at
     // every application: cycles stop at the inner target, the true residual decides
     const bool ml = use_ml && s->ml_on && !fp64;
     const bool fp32 = s->mixed && !fp64;
-    k_s_setup<<<1, 256, 0, st>>>(s->d_ks, s->d_part, VEC_GRID, tol, maxit,
+    k_s_setup<<<1, SUM_BS, 0, st>>>(s->d_ks, s->d_part, vv.terms, vv.per, tol, maxit,
                                  (fp32 || ml) ? MIXED_INNER : 0.0);
     count_launch(s, st);
     BO_LAUNCH_CHECK("bicgstab setup");
@@ -926,6 +995,8 @@ int run_bicgstab(bo_sim* s, double tol, int maxit, int* its, bool use_ml, bool f
     int prev_it = 0;
     for (int round = 0;; ++round) {
         if (loop) {
+            k_s1<<<1, 1, 0, st>>>(s->d_ks);
+            count_launch(s, st);
             graph_launch(s, s->g_loop, st);
         } else {
             replay_iterations(s, g, timed, &prev_it);
@@ -934,9 +1005,9 @@ int run_bicgstab(bo_sim* s, double tol, int maxit, int* its, bool use_ml, bool f
         // FP64 true residual r = b - Op x; accept, restart from it, or give up
         timer_begin(s, t_check);
         enqueue_op<3>(s, st, s->d_xs, s->d_r, s->d_b, nullptr);
-        k_s_restart<<<1, 256, 0, st>>>(s->d_ks, s->d_part, VEC_GRID, round < MAX_RESTARTS);
+        k_s_restart<<<1, SUM_BS, 0, st>>>(s->d_ks, s->d_part, vc.terms, vc.per, round < MAX_RESTARTS);
         count_launch(s, st);
-        k_restart_vectors<<<VEC_GRID, VEC_BS, 0, st>>>(N, s->d_r, s->d_rh, s->d_pk, s->d_v,
+        k_restart_vectors<<<vv.grid, vv.bs, 0, st>>>(N, s->d_r, s->d_rh, s->d_pk, s->d_v,
                                                        s->d_ks);
         count_launch(s, st);
         timer_end(s, t_check);
