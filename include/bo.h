@@ -507,7 +507,7 @@ bo_status bo_learn_enable(bo_sim* sim, int on);
  * BiCGStab residuals of its solve, until max_systems are kept or the device
  * has no room left; max_systems = 0 stops collecting and keeps the set.
  * Needs parameters (BO_ERR_STATE); with online training on, samples must be
- * its own count.  Memory: about 0.9 KB per cell plus 24 B per cell and
+ * its own count.  Memory: about 0.85 KB per cell plus 24 B per cell and
  * residual for every kept system.
  * bo_learn_set_info: the kept systems and residuals (either pointer may be
  * NULL).
