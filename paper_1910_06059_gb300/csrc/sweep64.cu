@@ -133,7 +133,7 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
                 if (l == NL || (known + RING <= l && (known = begun()) + RING <= l)) {
                     asm volatile("cp.async.wait_all;" ::: "memory");
                     __syncwarp();
-                    if (told != l && lane == 0) st_level(&s_copied, l);
+                    if (told != l && lane == 0) st_level_release(&s_copied, l);
                     told = l;
                     if (l == NL) break;
                     int q = 0;
@@ -170,7 +170,7 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
                 if (l == 0 && lane == 0) st_level(&s_begun, 1);
                 // the next level's entries (the first one's too) are in
                 const int last = min(l + 1, NL - 1);
-                for (q = 0; ld_level(&s_copied) <= last && ++q < WAIT_LIMIT;) {}
+                for (q = 0; ld_level_acquire(&s_copied) <= last && ++q < WAIT_LIMIT;) {}
                 if (q >= WAIT_LIMIT && lane == 0) atomicExch(a.err, 1);
                 __syncwarp();
                 level_arrive(l & (RING - 1));

@@ -16,9 +16,12 @@ static_assert(TSJ == 4 && TSK == 3, "one warp per j-line of the tile, three line
 __device__ __forceinline__ unsigned sa(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
-// Level counters in shared memory.  Plain volatile accesses: a warp's shared
-// memory accesses are performed in order, and a release would also wait for the
-// warp's global stores under way (several hundred cycles a level).
+// Level counters in shared memory.  Plain volatile accesses: such a counter only
+// says that a place may be overwritten.  Its store follows a barrier that every
+// reader of the place has passed (the reads are performed by then), and the writer
+// of the place has the counter's value before it issues its stores.  A release
+// would also wait for the warp's global stores under way (several hundred cycles a
+// level).
 __device__ __forceinline__ int ld_level(const int* p) {
     int v;
     asm volatile("ld.volatile.shared.b32 %0, [%1];" : "=r"(v) : "r"(sa(p)) : "memory");
@@ -26,6 +29,16 @@ __device__ __forceinline__ int ld_level(const int* p) {
 }
 __device__ __forceinline__ void st_level(int* p, int v) {
     asm volatile("st.volatile.shared.b32 [%0], %1;" ::"r"(sa(p)), "r"(v) : "memory");
+}
+// A counter that announces data: the writes that came before it (with a
+// __syncwarp, those of the whole warp) are seen by whoever reads the new value.
+__device__ __forceinline__ int ld_level_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(sa(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_level_release(int* p, int v) {
+    asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(sa(p)), "r"(v) : "memory");
 }
 // Opening of a level, on one of RING barriers in turn: its face warp arrives
 // (possibly several levels early), the compute warps wait.  The forms that
