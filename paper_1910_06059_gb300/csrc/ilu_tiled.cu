@@ -90,7 +90,7 @@ double* faceK3(bo_sim* s) {
 }
 
 void setup_sweeps(bo_sim* s) {
-    BO_CUDA(cudaMemset(s->d_sweep_sync, 0, sizeof(int) * 4));
+    BO_CUDA(cudaMemsetAsync(s->d_sweep_sync, 0, sizeof(int) * 4, s->stream));
     setup_sweeps64(s);
     setup_sweeps32(s);
 }

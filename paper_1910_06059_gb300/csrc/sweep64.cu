@@ -388,12 +388,13 @@ void reset_inbox(bo_sim* s, cudaStream_t st) {
 }
 
 // The tickets of a launch are counted from the last launch's with the same grid.
+// On the simulator's stream: the legacy stream has no order with a non-blocking one.
 void reset_tickets(bo_sim* s) {
-    BO_CUDA(cudaMemset(s->sweep.ticket, 0, 3 * sizeof(unsigned long long)));
+    BO_CUDA(cudaMemsetAsync(s->sweep.ticket, 0, 3 * sizeof(unsigned long long), s->stream));
 }
 
-// Plan of both sweeps for the current block-Jacobi boxes.  The new plan is
-// complete before the old one is given up.
+// Plan of both sweeps for the current block-Jacobi boxes, filled on the
+// simulator's stream.  The new plan is complete before the old one is given up.
 void setup_sweeps64(bo_sim* s) {
     const Geom& g = s->geo;
     SweepPlan p;
@@ -407,22 +408,23 @@ void setup_sweeps64(bo_sim* s) {
                 fail(BO_ERR_INVALID_ARG, "grid too large for the sweeps' 32-bit positions");
             auto alloc = [&](auto** q, size_t count) {
                 BO_CUDA(cudaMalloc(reinterpret_cast<void**>(q), sizeof(**q) * count));
-                BO_CUDA(cudaMemset(*q, 0, sizeof(**q) * count));   // idle slots stay zero
+                BO_CUDA(cudaMemsetAsync(*q, 0, sizeof(**q) * count, s->stream));   // idle slots stay zero
             };
             alloc(&p.tiles[d], o.tiles.size());
             alloc(&p.line[d], o.line.size());
             alloc(&p.S[d], lev * TSJ * 96);
             alloc(&p.Q[d], lev * SLOT);
-            BO_CUDA(cudaMemcpy(p.tiles[d], o.tiles.data(), sizeof(SweepTile) * o.tiles.size(),
-                               cudaMemcpyHostToDevice));
-            BO_CUDA(cudaMemcpy(p.line[d], o.line.data(), sizeof(unsigned) * o.line.size(),
-                               cudaMemcpyHostToDevice));
+            BO_CUDA(cudaMemcpyAsync(p.tiles[d], o.tiles.data(), sizeof(SweepTile) * o.tiles.size(),
+                                    cudaMemcpyHostToDevice, s->stream));
+            BO_CUDA(cudaMemcpyAsync(p.line[d], o.line.data(), sizeof(unsigned) * o.line.size(),
+                                    cudaMemcpyHostToDevice, s->stream));
             if (d == 0) {
                 alloc(&p.inbox, lev * FACE_W);
                 alloc(&p.inbox9, lev * FACE9_W);
                 alloc(&p.ticket, 3);
                 alloc(&p.Dn, 9 * (size_t)g.n);
             }
+            BO_CUDA(cudaStreamSynchronize(s->stream));   // the host arrays end here
         }
     } catch (...) {
         free_plan(p);
