@@ -515,6 +515,7 @@ bo_status bo_set_properties(bo_sim* s, const double* perm, const double* poro,
             BO_CUDA(cudaMemcpy(d_rw, rw.data(), sizeof(double) * s->nw, cudaMemcpyHostToDevice));
             BO_CUDA(cudaMemcpy(d_skin, skin.data(), sizeof(double) * s->nw, cudaMemcpyHostToDevice));
         }
+        wait_legacy_stream();
         launch_static(s);
         launch_wi(s, s->d_cellcon + n, d_rw, d_skin);
         sync(s);
@@ -1398,6 +1399,7 @@ bo_status bo_set_well_model(bo_sim* s, int model, int storage) {
                 w[q].vw = s->wells_h[q].vw = (full && storage) ? s->well_volume[q] : 0.0;
             }
             BO_CUDA(cudaMemcpy(s->d_wells, w.data(), sizeof(WellDev) * s->nw, cudaMemcpyHostToDevice));
+            wait_legacy_stream();
         }
         s->well_model = full ? BO_WELL_MODEL_STANDARD : BO_WELL_MODEL_REDUCED;
         s->well_storage = storage != 0;

@@ -25,6 +25,9 @@ bo_status set_last_error(bo_status st, const std::string& msg);   // returns st
 void check_cuda(cudaError_t e, const char* what, const char* file, int line);
 #define BO_CUDA(call) ::bo::check_cuda((call), #call, __FILE__, __LINE__)
 #define BO_LAUNCH_CHECK(name) ::bo::check_cuda(cudaGetLastError(), name, __FILE__, __LINE__)
+// After cudaMemset and cudaMemcpy of a set-up: they run on the legacy stream, which
+// has no order with a simulator's non-blocking one, and may return before they end.
+inline void wait_legacy_stream() { BO_CUDA(cudaStreamSynchronize(cudaStreamLegacy)); }
 
 // ---------------------------------------------------------------------------
 // Data layout in HBM (n cells, natural order c = i + nx*(j + ny*k)):

@@ -355,6 +355,7 @@ void cpr_build(bo_sim* s) {
     c->lv[0].x = c->x1;   // x1 = E_p x_p: its s_w and x columns stay zero
     c->r2 = dzeros<double>(3 * (size_t)n);
     c->status = dzeros<int>(1);
+    wait_legacy_stream();
 }
 
 void cpr_free(bo_sim* s) {

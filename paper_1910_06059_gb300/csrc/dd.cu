@@ -356,6 +356,7 @@ static void dd_setup(bo_sim* s) {
     zeros(&d->part, 2 * (size_t)d->K * DD_GX);
     zeros(&d->red, 2);
     zeros(&d->sop, std::max(s->nw, 1));
+    wait_legacy_stream();
 }
 
 int dd_bicgstab(bo_sim* s, double tol, int maxit, int* its) {

@@ -508,6 +508,7 @@ void std_wells_setup(bo_sim* s) {
         BO_CUDA(cudaMemset(s->d_wB4, 0, sizeof(double) * 12 * s->ncon));
         BO_CUDA(cudaMemset(s->d_wC4, 0, sizeof(double) * 12 * s->ncon));
         BO_CUDA(cudaMemset(s->d_wcorr, 0, sizeof(double) * 3 * s->ncon));
+        wait_legacy_stream();
     }
 }
 
