@@ -1318,10 +1318,6 @@ bo_status bo_set_solve_schedule(bo_sim* s, int kind) {
         need(kind == BO_SCHEDULE_TILED || kind == BO_SCHEDULE_BLOCK, BO_ERR_INVALID_ARG,
              "bo_set_solve_schedule: kind must be BO_SCHEDULE_TILED or BO_SCHEDULE_BLOCK");
         s->solve_schedule = kind;
-        if (kind == BO_SCHEDULE_BLOCK && s->factored) {
-            need_tile_factors(s);
-            enqueue_tile_factors(s, s->stream);
-        }
     });
 }
 

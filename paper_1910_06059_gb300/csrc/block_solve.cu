@@ -426,6 +426,7 @@ k_block_bicgstab(BlockArgs a) {
 // Host side
 // ---------------------------------------------------------------------------
 static BlockArgs block_args(bo_sim* s) {
+    current_tile_factors(s);
     BlockArgs a{};
     a.g = s->geo;
     a.NJ = (s->geo.ny + TJ - 1) / TJ;

@@ -193,6 +193,7 @@ struct bo_sim {
     double* d_R = nullptr;       // 3n
     double* d_A = nullptr;       // 63n
     double* d_P = nullptr;       // 63 x tile-order ILU(0) data (FP32 sweeps, one-CTA solve; at need)
+    bool tile_valid = false;     // d_P holds the current factors (kept for the one-CTA solve)
     bo::SweepPlan sweep;         // FP64 sweeps: tiles, factors, right-hand sides
     float* d_P32 = nullptr;      // FP32 factors in the FP32 sweep layout (mixed mode)
     float* d_r32 = nullptr;      // FP32 sweep input, tile order (mixed mode)
@@ -312,6 +313,7 @@ void free_sweeps64(bo_sim* s);
 void reset_tickets(bo_sim* s);                   // after a change of the sweeps' grid
 void enqueue_scaled_factors(bo_sim* s, cudaStream_t st); // both sweeps' blocks from A and D^-1
 void need_tile_factors(bo_sim* s);               // the tile-order buffer d_P
+void current_tile_factors(bo_sim* s);            // d_P holds the current factors after this
 void enqueue_tile_factors(bo_sim* s, cudaStream_t st);   // gathers d_P from the factorisation
 size_t face_storage(const bo_sim* s);
 void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad);

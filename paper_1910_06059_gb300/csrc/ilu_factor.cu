@@ -279,6 +279,7 @@ void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad) {
 }
 
 void enqueue_scaled_factors(bo_sim* s, cudaStream_t st) {
+    s->tile_valid = false;
     enqueue_scaled<0>(s, st);
     enqueue_scaled<1>(s, st);
 }

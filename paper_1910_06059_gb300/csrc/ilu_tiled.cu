@@ -109,6 +109,15 @@ void enqueue_tile_factors(bo_sim* s, cudaStream_t st) {
     BO_LAUNCH_CHECK("k_tile_factors");
 }
 
+// For the one-CTA solve, at its launch: what it reads is gathered once for every
+// factorisation that it is used with, and for none that it is not.
+void current_tile_factors(bo_sim* s) {
+    if (s->tile_valid) return;
+    need_tile_factors(s);
+    enqueue_tile_factors(s, s->stream);
+    s->tile_valid = true;
+}
+
 // Sentinels of the current precision's sweeps (after a precision switch or an
 // abandoned sweep).
 void reset_sweep_faces(bo_sim* s) {

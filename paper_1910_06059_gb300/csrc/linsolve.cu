@@ -848,10 +848,7 @@ void launch_factor(bo_sim* s) {
     timer_begin(s, t);
     graph_launch(s, s->g_factor, s->stream);
     timer_end(s, t);
-    if (s->solve_schedule == BO_SCHEDULE_BLOCK && !s->mixed) {   // the one-CTA solve's data
-        need_tile_factors(s);
-        enqueue_tile_factors(s, s->stream);
-    }
+    s->tile_valid = false;
 }
 
 void launch_precond(bo_sim* s, const double* r, double* z) {

@@ -432,6 +432,7 @@ void setup_sweeps64(bo_sim* s) {
     }
     free_plan(s->sweep);
     s->sweep = p;
+    s->tile_valid = false;
     // four CTAs on an SM need 144 KB of shared memory
     for (const void* k : {(const void*)k_sweep<true>, (const void*)k_sweep<false>})
         BO_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
