@@ -24,6 +24,7 @@ bo_status set_last_error(bo_status st, const std::string& msg) {
 
 void check_cuda(cudaError_t e, const char* what, const char* file, int line) {
     if (e == cudaSuccess) return;
+    (void)cudaGetLastError();   // reported here: the next launch check must not find it again
     std::string m = std::string(what) + ": " + cudaGetErrorString(e) + " (" + file + ":" +
                     std::to_string(line) + ")";
     fail(e == cudaErrorMemoryAllocation ? BO_ERR_OOM : BO_ERR_CUDA, m);

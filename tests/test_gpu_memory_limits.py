@@ -1,0 +1,64 @@
+"""Calls that the device has no room for: they fail with BO_ERR_OOM and leave the
+simulator as it was.  The device is filled with one torch allocation for the call.
+
+Bar: the same bits before and after."""
+from __future__ import annotations
+
+import contextlib
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+    from paper_1910_06059_gb300.build import build
+    build()
+
+
+@contextlib.contextmanager
+def _room(megabytes):
+    """Leaves about this much free on the device."""
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - (megabytes << 20), dtype=torch.uint8,
+                         device="cuda")
+    try:
+        yield
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+
+
+def _factored(shape):
+    from paper_1910_06059_gb300 import Sim
+    m = synth.small_model(*shape, wells="5spot")
+    g = Sim(m)
+    g.set_state(*synth.random_state(m, seed_member=4))
+    g.begin_step()
+    g.assemble(2.0 * synth.DAY)
+    g.factor()
+    return g, np.random.default_rng(6).normal(size=3 * g.n)
+
+
+def test_an_error_is_reported_once():
+    """The one-CTA solve's factors (144 MB) do not fit; the next call on the thread
+    succeeds."""
+    from paper_1910_06059_gb300 import _lib
+    g, r = _factored((60, 64, 64))
+    z = g.precond_apply(r)
+    g.solve_schedule = "block"
+    with _room(64), pytest.raises(_lib.BoError, match="OOM"):
+        g.precond_apply(r)
+    g.solve_schedule = "tiled"
+    assert np.array_equal(g.precond_apply(r), z)
+    g.close()
