@@ -1157,7 +1157,8 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
         double first = 0.0, last = 0.0;
         long long cnt = 0;
         // each kept system's Jacobian, pivot inverses, features and scalings take
-        // the place of the current ones while its residuals are trained on
+        // the place of the current ones while its residuals are trained on; the
+        // current system, with the blocks made from it, is back on every way out
         struct Swap {
             bo_sim* s;
             double *A, *Dn;
@@ -1168,6 +1169,12 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
                 s->sweep.Dn = Dn;
                 s->d_ml_featf = featf;
                 s->d_ml_cell = cell;
+                if (!s->factored) return;
+                try {
+                    enqueue_scaled_factors(s, s->stream);
+                } catch (...) {
+                    s->factored = false;   // the blocks are a kept system's
+                }
             }
         };
         {
@@ -1190,7 +1197,6 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
             }
         }
         }
-        if (s->factored) enqueue_scaled_factors(s, s->stream);
         sync(s);
         check_timeout(s);
         s->ml_train_ms +=

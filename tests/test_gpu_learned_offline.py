@@ -96,3 +96,31 @@ def test_one_cta_schedule_holds_its_factors_only_where_it_runs():
         g.close()
     assert counts[0] == counts[1]
     assert free[1] <= free[0] + (8 << 20)   # the tile-order factors are 70 MB
+
+
+def test_failed_training_leaves_the_current_factors():
+    """The device has no room for the one-CTA solve's factors (144 MB), so the call fails
+    on its first kept system; the factorisation made before still applies."""
+    from paper_1910_06059_gb300 import _lib
+    g = _collected((60, 64, 64), systems=1)
+    g.begin_step()
+    g.assemble(30.0 * synth.DAY)
+    g.factor()
+    r = np.random.default_rng(3).normal(size=3 * g.n)
+    z = g.precond_apply(r)
+    g.learn_set_params(synth.learned_init(0))
+    g.solve_schedule = "block"
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - (64 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(_lib.BoError):
+            g.learn_train_offline(epochs=1, lr=1e-30)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    g.solve_schedule = "tiled"
+    assert np.array_equal(g.precond_apply(r), z)
+    g.solve_schedule = "block"
+    first, _ = g.learn_train_offline(epochs=1, lr=1e-30)
+    assert np.isfinite(first)
+    g.close()
