@@ -186,6 +186,8 @@ static void learn_store_system(bo_sim* s) {
         return;
     }
     q.nr = nr;
+    q.ysub = s->ysub;
+    q.zsub = s->zsub;
     BO_CUDA(cudaMemcpyAsync(q.A, s->d_A, sizeof(double) * NA, cudaMemcpyDeviceToDevice, s->stream));
     BO_CUDA(cudaMemcpyAsync(q.Dn, s->sweep.Dn, sizeof(double) * ND, cudaMemcpyDeviceToDevice, s->stream));
     BO_CUDA(cudaMemcpyAsync(q.featf, s->d_ml_featf, sizeof(float) * 64 * n, cudaMemcpyDeviceToDevice,
@@ -1171,7 +1173,7 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
                 s->d_ml_cell = cell;
                 if (!s->factored) return;
                 try {
-                    enqueue_scaled_factors(s, s->stream);
+                    enqueue_scaled_factors(s, s->stream, s->ysub, s->zsub);
                 } catch (...) {
                     s->factored = false;   // the blocks are a kept system's
                 }
@@ -1185,7 +1187,8 @@ bo_status bo_learn_train_offline(bo_sim* s, int epochs, double lr, double* first
                 s->sweep.Dn = q.Dn;
                 s->d_ml_featf = q.featf;
                 s->d_ml_cell = q.cell;
-                enqueue_scaled_factors(s, s->stream);
+                // the boxes of its pivots, whatever boxes are set now
+                enqueue_scaled_factors(s, s->stream, q.ysub, q.zsub);
                 for (int j = 0; j < q.nr; ++j) {
                     const double L = learn_loss_grad(s, q.r + (size_t)j * N);
                     if (ep == 0) first += L;

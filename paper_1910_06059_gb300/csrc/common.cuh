@@ -119,7 +119,7 @@ struct EagerTimer {
 
 // One Newton system kept for offline training of the learned stage: its
 // Jacobian, pivot inverses, FP32 features, per-cell scalings and nr residuals
-// of its BiCGStab solve ([nr][3n]).
+// of its BiCGStab solve ([nr][3n]), and the block-Jacobi boxes of its factorisation.
 struct LearnSystem {
     double* A = nullptr;
     double* Dn = nullptr;
@@ -127,6 +127,7 @@ struct LearnSystem {
     float4* cell = nullptr;
     double* r = nullptr;
     int nr = 0;
+    int ysub = 0, zsub = 0;
 };
 
 // FP64 sweeps (sweep64.cu): a tile of TSJ x TSK x-lines in one sweep direction
@@ -311,7 +312,8 @@ void read_flags_async(bo_sim* s);   // h_flags, valid after the next wait for th
 void setup_sweeps64(bo_sim* s);                  // FP64 sweep plan for the current boxes
 void free_sweeps64(bo_sim* s);
 void reset_tickets(bo_sim* s);                   // after a change of the sweeps' grid
-void enqueue_scaled_factors(bo_sim* s, cudaStream_t st); // both sweeps' blocks from A and D^-1
+// both sweeps' blocks from A and D^-1, cut at the boundaries of these boxes too
+void enqueue_scaled_factors(bo_sim* s, cudaStream_t st, int ysub, int zsub);
 void need_tile_factors(bo_sim* s);               // the tile-order buffer d_P
 void current_tile_factors(bo_sim* s);            // d_P holds the current factors after this
 void enqueue_tile_factors(bo_sim* s, cudaStream_t st);   // gathers d_P from the factorisation

@@ -213,12 +213,13 @@ k_factor_wave(SweepArgs a, const double* __restrict__ A, const unsigned* __restr
 // -x, -y, -z; 1: +x, +y, +z) in its lane order: a warp a line of tiles' jj and
 // CHUNK levels (a 32-byte sector of A holds four cells of a line, so the levels
 // of a chunk share them), 27 lanes (kk, row, d), three entries a lane.  Idle
-// places keep the zeros they were allocated with.
+// places keep the zeros they were allocated with.  Couplings that leave a box of the
+// plan, or of cy x cz lines (0: no cut), are left out.
 constexpr int CHUNK = 8;
 template <int DIR>
 __global__ void __launch_bounds__(256)
 k_scaled_blocks(SweepArgs a, const double* __restrict__ A, const double* __restrict__ Dn,
-                double* __restrict__ S) {
+                double* __restrict__ S, int cy, int cz) {
     const int lane = threadIdx.x & 31, chunks = (a.NL + CHUNK - 1) / CHUNK;
     const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const int jj = (int)(w % TSJ), ch = (int)(w / TSJ % chunks);
@@ -229,7 +230,9 @@ k_scaled_blocks(SweepArgs a, const double* __restrict__ A, const double* __restr
     if (jj >= t.nj || kk >= t.nk) return;
     const int js = t.j0 + jj, ks = t.k0 + kk;
     const int j = DIR ? a.g.ny - 1 - js : js, k = DIR ? a.g.nz - 1 - ks : ks;
-    const bool keep = d == 0 || (d == 1 ? jj > 0 || t.depJ : kk > 0 || t.depK);
+    const int cut = d == 1 ? cy : cz;
+    const bool keep = d == 0 || ((d == 1 ? jj > 0 || t.depJ : kk > 0 || t.depK) &&
+                                 (cut == 0 || ((d == 1 ? j : k) + DIR) % cut != 0));
     const int blk = 1 + 2 * d + DIR;   // NB_MX, NB_PX, NB_MY, ... in turn
     static_assert(NB_MX == 1 && NB_PX == 2 && NB_MY == 3 && NB_PY == 4 && NB_MZ == 5 && NB_PZ == 6,
                   "block numbers");
@@ -254,11 +257,11 @@ k_scaled_blocks(SweepArgs a, const double* __restrict__ A, const double* __restr
 // Host side
 // ---------------------------------------------------------------------------
 template <int DIR>
-static void enqueue_scaled(bo_sim* s, cudaStream_t st) {
+static void enqueue_scaled(bo_sim* s, cudaStream_t st, int cy = 0, int cz = 0) {
     const SweepPlan& p = s->sweep;
     const long long warps = (long long)p.T * TSJ * ((p.NL + CHUNK - 1) / CHUNK);
     k_scaled_blocks<DIR><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(sweep_args(s, DIR), s->d_A,
-                                                                     p.Dn, p.S[DIR]);
+                                                                     p.Dn, p.S[DIR], cy, cz);
     count_launch(s, st);
     BO_LAUNCH_CHECK("k_scaled_blocks");
 }
@@ -278,10 +281,10 @@ void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad) {
     }
 }
 
-void enqueue_scaled_factors(bo_sim* s, cudaStream_t st) {
+void enqueue_scaled_factors(bo_sim* s, cudaStream_t st, int ysub, int zsub) {
     s->tile_valid = false;
-    enqueue_scaled<0>(s, st);
-    enqueue_scaled<1>(s, st);
+    enqueue_scaled<0>(s, st, ysub, zsub);
+    enqueue_scaled<1>(s, st, ysub, zsub);
 }
 
 // D^-1 of every cell, [n][9].

@@ -124,3 +124,16 @@ def test_failed_training_leaves_the_current_factors():
     first, _ = g.learn_train_offline(epochs=1, lr=1e-30)
     assert np.isfinite(first)
     g.close()
+
+
+@pytest.mark.parametrize("boxes", [(0, 0), (16, 0), (0, 8), (16, 8)])
+def test_kept_systems_keep_their_boxes(boxes):
+    """A set collected with 8 x 4-line boxes has one preconditioner, whatever coarser
+    boxes are set when it is trained on."""
+    def narrow(g):
+        g.subdomains, g.subdomains_z = 8, 4
+    g = _collected((14, 21, 13), before=narrow)
+    want = _loss(g)
+    g.subdomains, g.subdomains_z = boxes
+    assert np.isclose(_loss(g), want, rtol=RTOL)
+    g.close()
