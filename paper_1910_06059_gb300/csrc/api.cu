@@ -85,7 +85,7 @@ static void free_all(bo_sim* s) {
                     s->d_props, s->d_R, s->d_A, s->d_P, s->d_face, s->d_cellcon, s->d_wells,
                     s->d_con_cell, s->d_con_wi, s->d_wB, s->d_wC, s->d_b, s->d_xs, s->d_r,
                     s->d_rh, s->d_pk, s->d_v, s->d_s, s->d_t, s->d_ph, s->d_sh, s->d_part,
-                    s->d_ks, s->d_ns, s->d_sweep_sync, s->d_P32, s->d_r32, s->d_y32,
+                    s->d_ks, s->d_ns, s->d_sweep_sync, s->d_P32, s->d_D32, s->d_r32, s->d_y32,
                     s->d_ml_theta, s->d_ml_grad, s->d_ml_m, s->d_ml_v, s->d_ml_wbf,
                     s->d_ml_feat, s->d_ml_featf, s->d_ml_cell, s->d_ml_part, s->d_ml_delta,
                     s->d_ml_u, s->d_ml_z0, s->d_ml_e, s->d_ml_dd, s->d_ml_scal, s->d_ml_count,
@@ -950,15 +950,12 @@ bo_status bo_set_precision(bo_sim* s, int precision) {
         sync(s);
         if (mixed && s->d_P32 == nullptr) {
             dalloc(&s->d_P32, factors32_floats(s));
+            dalloc(&s->d_D32, dinv32_doubles(s));
             dalloc(&s->d_r32, vec32_floats(s));
             dalloc(&s->d_y32, vec32_floats(s));
         }
         s->mixed = mixed;
-        if (mixed) {   // factors of an earlier bo_factor stay usable
-            need_tile_factors(s);
-            enqueue_tile_factors(s, s->stream);
-            convert_factors32(s, s->stream);
-        }
+        if (mixed) convert_factors32(s, s->stream);   // factors of an earlier bo_factor stay usable
         reset_sweep_faces(s);
         build_graphs(s);
         sync(s);

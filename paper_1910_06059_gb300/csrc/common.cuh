@@ -37,7 +37,7 @@ inline void wait_legacy_stream() { BO_CUDA(cudaStreamSynchronize(cudaStreamLegac
 //     e = 3*r + s for dR_r,c / dy_s,neighbour(b); zero where no neighbour.
 //   ILU(0): D^-1 [9][n] in natural order and the scaled blocks D^-1 A in the
 //     sweeps' lane orders (see tiles.cuh); P gathers them in the tile order of
-//     the FP32 sweeps and the one-CTA solve (pidx).
+//     the one-CTA solve (pidx).
 // ---------------------------------------------------------------------------
 enum { NB_DIAG = 0, NB_MX = 1, NB_PX = 2, NB_MY = 3, NB_PY = 4, NB_MZ = 5, NB_PZ = 6 };
 constexpr int NPROP = 28;   // per-cell face quantities: rho_a, b_a lam_a (3 x 4), r_go b_o lam_o (4)
@@ -193,10 +193,11 @@ struct bo_sim {
     double* d_props = nullptr;   // NPROP * n
     double* d_R = nullptr;       // 3n
     double* d_A = nullptr;       // 63n
-    double* d_P = nullptr;       // 63 x tile-order ILU(0) data (FP32 sweeps, one-CTA solve; at need)
-    bool tile_valid = false;     // d_P holds the current factors (kept for the one-CTA solve)
+    double* d_P = nullptr;       // 63 x tile-order ILU(0) data (one-CTA solve; at need)
+    bool tile_valid = false;     // d_P holds the current factors
     bo::SweepPlan sweep;         // FP64 sweeps: tiles, factors, right-hand sides
     float* d_P32 = nullptr;      // FP32 factors in the FP32 sweep layout (mixed mode)
+    double* d_D32 = nullptr;     // D^-1 in FP64 in its tile order (mixed mode)
     float* d_r32 = nullptr;      // FP32 sweep input, tile order (mixed mode)
     float* d_y32 = nullptr;      // FP32 sweep work vector, tile order (mixed mode)
     bool mixed = false;          // preconditioner applies in FP32
@@ -314,15 +315,14 @@ void free_sweeps64(bo_sim* s);
 void reset_tickets(bo_sim* s);                   // after a change of the sweeps' grid
 // both sweeps' blocks from A and D^-1, cut at the boundaries of these boxes too
 void enqueue_scaled_factors(bo_sim* s, cudaStream_t st, int ysub, int zsub);
-void need_tile_factors(bo_sim* s);               // the tile-order buffer d_P
 void current_tile_factors(bo_sim* s);            // d_P holds the current factors after this
-void enqueue_tile_factors(bo_sim* s, cudaStream_t st);   // gathers d_P from the factorisation
 size_t face_storage(const bo_sim* s);
 void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad);
 void enqueue_fwd(bo_sim* s, cudaStream_t st, const double* r, double* y, const KrylovScalars* ks);
 void enqueue_bwd(bo_sim* s, cudaStream_t st, double* z, const KrylovScalars* ks);
 void export_dinv(bo_sim* s, double* dinv);
 size_t factors32_floats(const bo_sim* s);        // size of d_P32 (FP32 sweep layout)
+size_t dinv32_doubles(const bo_sim* s);          // size of d_D32
 size_t vec32_floats(const bo_sim* s);            // size of d_r32, d_y32 (tile order)
 void convert_factors32(bo_sim* s, cudaStream_t st);
 void reset_sweep_faces(bo_sim* s);                // sentinels of the current precision

@@ -275,10 +275,7 @@ void enqueue_factor(bo_sim* s, cudaStream_t st, int* bad) {
     count_launch(s, st);
     BO_LAUNCH_CHECK("k_factor_wave");
     enqueue_scaled<0>(s, st);
-    if (s->mixed) {
-        enqueue_tile_factors(s, st);
-        convert_factors32(s, st);
-    }
+    if (s->mixed) convert_factors32(s, st);
 }
 
 void enqueue_scaled_factors(bo_sim* s, cudaStream_t st, int ysub, int zsub) {

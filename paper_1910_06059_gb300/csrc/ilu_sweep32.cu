@@ -363,36 +363,6 @@ k_bwd32(TileArgs a, const float4* __restrict__ B, float4* __restrict__ Yt, float
 // ---------------------------------------------------------------------------
 // Layout conversions (bulk, all lanes busy)
 // ---------------------------------------------------------------------------
-// FP64 factors (tile order, pidx) -> FP32 chunks F (blocks 1-3) and B
-// (blocks 4-6).
-__global__ void k_factors32(const double* __restrict__ P, size_t NP, float4* __restrict__ F,
-                            float4* __restrict__ Bk) {
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < NP;
-         q += (size_t)gridDim.x * blockDim.x) {
-        const size_t s = q >> 5;
-        const int lane = (int)(q & 31);
-        auto Pq = [&](int e) { return P[pidx(s, e, lane)]; };
-#pragma unroll
-        for (int g = 0; g < FWD_G; ++g) {
-            float4 v;
-            v.x = (float)Pq(9 + 4 * g);
-            v.y = (float)Pq(9 + 4 * g + 1);
-            v.z = (float)Pq(9 + 4 * g + 2);
-            v.w = (g < FWD_G - 1) ? (float)Pq(9 + 4 * g + 3) : 0.f;
-            F[(s * FWD_G + g) * 32 + lane] = v;
-        }
-#pragma unroll
-        for (int g = 0; g < BWD_G; ++g) {
-            float4 v;
-            v.x = (float)Pq(36 + 4 * g);
-            v.y = (float)Pq(36 + 4 * g + 1);
-            v.z = (float)Pq(36 + 4 * g + 2);
-            v.w = (g < BWD_G - 1) ? (float)Pq(36 + 4 * g + 3) : 0.f;
-            Bk[(s * BWD_G + g) * 32 + lane] = v;
-        }
-    }
-}
-
 // Thread g of the conversions handles line (t, lane) at level l, g = (t*32 + lane)*NL + l,
 // so neighbouring threads touch neighbouring cells of one x-line.
 __device__ __forceinline__ bool line_cell(const TileArgs& a, size_t g, size_t& slot, int& c) {
@@ -420,9 +390,39 @@ __device__ __forceinline__ bool slot_cell(const TileArgs& a, size_t q, int& c) {
     return true;
 }
 
-// Q = D^-1 r in FP64 (r[e*n + c], D^-1 = block 0 of the FP64 factors), rounded
-// into the FP32 tile-order vector; slots without a cell get zeros.
-__global__ void k_to_tiles32(TileArgs a, const double* __restrict__ P, const double* __restrict__ r,
+// Factorisation -> FP32 chunks F (lower blocks) and B (upper blocks) and, in FP64,
+// D^-1 in the same tile order; slots without a cell get zeros.
+__global__ void k_factors32(TileArgs a, SweepFactors f, float4* __restrict__ F,
+                            float4* __restrict__ Bk, double* __restrict__ D) {
+    static_assert(FWD_G == 7 && BWD_G == 7, "27 entries in float4 groups");
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < a.NP;
+         q += (size_t)gridDim.x * blockDim.x) {
+        const size_t s = q >> 5;
+        const int lane = (int)(q & 31);
+        int c = 0;
+        const bool cell = slot_cell(a, q, c);
+        const int i = c % a.g.nx;
+        const double *lo = lower_blocks(f, c / a.g.nx, i), *up = upper_blocks(f, c / a.g.nx, i);
+        // entry q = 9 d + 3 row + s of a chunk
+        auto entry = [&](const double* b, int e) {
+            return cell && e < 27 ? (float)b[lane_entry(e % 9 / 3, e % 3, e / 9)] : 0.f;
+        };
+#pragma unroll
+        for (int g = 0; g < FWD_G; ++g) {
+            F[(s * FWD_G + g) * 32 + lane] = make_float4(entry(lo, 4 * g), entry(lo, 4 * g + 1),
+                                                         entry(lo, 4 * g + 2), entry(lo, 4 * g + 3));
+            Bk[(s * BWD_G + g) * 32 + lane] = make_float4(entry(up, 4 * g), entry(up, 4 * g + 1),
+                                                          entry(up, 4 * g + 2), entry(up, 4 * g + 3));
+        }
+#pragma unroll
+        for (int e = 0; e < 9; ++e)
+            D[(s * 9 + e) * 32 + lane] = cell ? f.Dn[(size_t)e * a.g.n + c] : 0.0;
+    }
+}
+
+// Q = D^-1 r in FP64 (r[e*n + c], D of k_factors32), rounded into the FP32
+// tile-order vector; slots without a cell get zeros.
+__global__ void k_to_tiles32(TileArgs a, const double* __restrict__ D, const double* __restrict__ r,
                              float4* __restrict__ V, const KrylovScalars* __restrict__ ks) {
     if (ks_skip_t(ks)) return;
     const size_t NP = a.NP;
@@ -434,11 +434,11 @@ __global__ void k_to_tiles32(TileArgs a, const double* __restrict__ P, const dou
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (slot_cell(a, q, c)) {
             const double r0 = r[c], r1 = r[(size_t)n + c], r2 = r[2 * (size_t)n + c];
+            const double* Dc = D + (q >> 5) * 288 + lane;
             double o[3];
 #pragma unroll
             for (int e = 0; e < 3; ++e)
-                o[e] = fma(P[pidx(q >> 5, 3 * e, lane)], r0,
-                           fma(P[pidx(q >> 5, 3 * e + 1, lane)], r1, P[pidx(q >> 5, 3 * e + 2, lane)] * r2));
+                o[e] = fma(Dc[96 * e], r0, fma(Dc[96 * e + 32], r1, Dc[96 * e + 64] * r2));
             v.x = (float)o[0];
             v.y = (float)o[1];
             v.z = (float)o[2];
@@ -479,6 +479,7 @@ size_t factors32_floats(const bo_sim* s) {
     TileArgs a = tile_args(s);
     return (size_t)a.T * a.NL * 32 * 4 * (FWD_G + BWD_G);
 }
+size_t dinv32_doubles(const bo_sim* s) { return 9 * tile_args(s).NP; }
 size_t vec32_floats(const bo_sim* s) {
     TileArgs a = tile_args(s);
     return (size_t)a.T * a.NL * 32 * 4;
@@ -512,7 +513,8 @@ void setup_sweeps32(bo_sim* s) {
 
 void convert_factors32(bo_sim* s, cudaStream_t st) {
     TileArgs a = tile_args(s);
-    k_factors32<<<152 * 8, 256, 0, st>>>(s->d_P, a.NP, fwd_factors(s), bwd_factors(s));
+    k_factors32<<<152 * 8, 256, 0, st>>>(a, sweep_factors(s), fwd_factors(s), bwd_factors(s),
+                                         s->d_D32);
     count_launch(s, st);
     BO_LAUNCH_CHECK("k_factors32");
 }
@@ -528,7 +530,7 @@ void enqueue_fwd32(bo_sim* s, cudaStream_t st, const double* r, const KrylovScal
     TileArgs a = tile_args(s);
     float4* R = reinterpret_cast<float4*>(s->d_r32);
     float4* Y = reinterpret_cast<float4*>(s->d_y32);
-    k_to_tiles32<<<152 * 8, 256, 0, st>>>(a, (const double*)s->d_P, r, R, ks);
+    k_to_tiles32<<<152 * 8, 256, 0, st>>>(a, (const double*)s->d_D32, r, R, ks);
     count_launch(s, st);
     launch_coop(st, a.T, 32, k_fwd32, a, (const float4*)fwd_factors(s), (const float4*)R, Y,
                 faceJ3f(s), faceK3f(s), ks);

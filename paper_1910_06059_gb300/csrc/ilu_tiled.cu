@@ -1,7 +1,6 @@
-// ILU(0) data in the 8 x 4-line tile order that the FP32 sweeps (ilu_sweep32.cu)
-// and the one-CTA solve (block_solve.cu) read, gathered from the factorisation
-// when one of them is selected; the dispatch of the sweeps by precision; the
-// bounded wait's self-test.
+// ILU(0) data in the 8 x 4-line tile order that the one-CTA solve (block_solve.cu)
+// reads, gathered from the factorisation at its launch; the dispatch of the sweeps
+// by precision; the bounded wait's self-test.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -23,16 +22,14 @@ k_tile_factors(TileArgs a, SweepFactors f, double* __restrict__ P) {
         const int j = t % a.NJ * TJ + jj, k = t / a.NJ * TK + kk, i = l - jj - kk;
         if (j >= a.g.ny || k >= a.g.nz || i < 0 || i >= a.g.nx) continue;
         const size_t jk = j + (size_t)a.g.ny * k, c = i + (size_t)a.g.nx * jk;
-        const unsigned pf = f.fline[jk], pb = f.bline[jk], qf = pf % 36 / 3, qb = pb % 36 / 3;
-        const double* sf = f.F + ((size_t)(pf / 36 + i) * TSJ + qf / TSK) * 96 + qf % TSK * 9;
-        const double* sb = f.B + ((size_t)(pb / 36 - i) * TSJ + qb / TSK) * 96 + qb % TSK * 9;
+        const double *lo = lower_blocks(f, jk, i), *up = upper_blocks(f, jk, i);
 #pragma unroll
         for (int e = 0; e < 9; ++e) {
             P[pidx(tl, e, lane)] = f.Dn[(size_t)e * a.g.n + c];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                P[pidx(tl, 9 + 9 * d + e, lane)] = sf[e % 3 * 32 + e / 3 * 3 + d];
-                P[pidx(tl, 36 + 9 * d + e, lane)] = sb[e % 3 * 32 + e / 3 * 3 + d];
+                P[pidx(tl, 9 + 9 * d + e, lane)] = lo[lane_entry(e / 3, e % 3, d)];
+                P[pidx(tl, 36 + 9 * d + e, lane)] = up[lane_entry(e / 3, e % 3, d)];
             }
         }
     }
@@ -95,26 +92,19 @@ void setup_sweeps(bo_sim* s) {
     setup_sweeps32(s);
 }
 
-// The tile-order buffer, made at its first use (not while a stream is captured).
-void need_tile_factors(bo_sim* s) {
-    if (s->d_P) return;
-    const size_t bytes = sizeof(double) * NPE * tile_args(s).NP;
-    BO_CUDA(cudaMalloc(reinterpret_cast<void**>(&s->d_P), bytes));
-    BO_CUDA(cudaMemsetAsync(s->d_P, 0, bytes, s->stream));
-}
-
-void enqueue_tile_factors(bo_sim* s, cudaStream_t st) {
-    k_tile_factors<<<152 * 8, 256, 0, st>>>(tile_args(s), sweep_factors(s), s->d_P);
-    count_launch(s, st);
-    BO_LAUNCH_CHECK("k_tile_factors");
-}
-
 // For the one-CTA solve, at its launch: what it reads is gathered once for every
 // factorisation that it is used with, and for none that it is not.
 void current_tile_factors(bo_sim* s) {
     if (s->tile_valid) return;
-    need_tile_factors(s);
-    enqueue_tile_factors(s, s->stream);
+    const TileArgs a = tile_args(s);
+    if (!s->d_P) {
+        const size_t bytes = sizeof(double) * NPE * a.NP;
+        BO_CUDA(cudaMalloc(reinterpret_cast<void**>(&s->d_P), bytes));
+        BO_CUDA(cudaMemsetAsync(s->d_P, 0, bytes, s->stream));   // idle places
+    }
+    k_tile_factors<<<152 * 8, 256, 0, s->stream>>>(a, sweep_factors(s), s->d_P);
+    count_launch(s, s->stream);
+    BO_LAUNCH_CHECK("k_tile_factors");
     s->tile_valid = true;
 }
 

@@ -128,6 +128,17 @@ struct SweepFactors {
     const unsigned *fline, *bline;
     double *F, *B, *Dn;           // S of both directions, D^-1 [9][n] in natural order
 };
+// The scaled lower (-x, -y, -z) and upper blocks of cell (i, j, k), jk = j + ny k:
+// entry (row, s) towards neighbour d at [lane_entry(row, s, d)].
+__device__ __forceinline__ const double* lower_blocks(const SweepFactors& f, size_t jk, int i) {
+    const unsigned p = f.fline[jk], line = p % 36 / 3;
+    return f.F + ((size_t)(p / 36 + i) * TSJ + line / TSK) * 96 + line % TSK * 9;
+}
+__device__ __forceinline__ const double* upper_blocks(const SweepFactors& f, size_t jk, int i) {
+    const unsigned p = f.bline[jk], line = p % 36 / 3;
+    return f.B + ((size_t)(p / 36 - i) * TSJ + line / TSK) * 96 + line % TSK * 9;
+}
+__host__ __device__ constexpr int lane_entry(int row, int s, int d) { return 32 * s + 3 * row + d; }
 struct SweepOrder {
     int T;
     std::vector<SweepTile> tiles;
@@ -144,7 +155,7 @@ void enqueue_bwd64(bo_sim* s, cudaStream_t st, double* z, const KrylovScalars* k
 
 // FP32 sweeps of the mixed-precision solver (ilu_sweep32.cu)
 void setup_sweeps32(bo_sim* s);                              // attributes, residency check
-void convert_factors32(bo_sim* s, cudaStream_t st);          // d_P -> FP32 sweep layout
+void convert_factors32(bo_sim* s, cudaStream_t st);          // factorisation -> FP32 sweep layout
 void enqueue_fwd32(bo_sim* s, cudaStream_t st, const double* r, const KrylovScalars* ks);
 void enqueue_bwd32(bo_sim* s, cudaStream_t st, double* z, const KrylovScalars* ks);
 void reset_faces32(bo_sim* s, cudaStream_t st);

@@ -62,3 +62,21 @@ def test_an_error_is_reported_once():
     g.solve_schedule = "tiled"
     assert np.array_equal(g.precond_apply(r), z)
     g.close()
+
+
+@pytest.mark.parametrize("shape", [(60, 64, 64), (31, 41, 50)])
+def test_mixed_precision_holds_its_factors_once(shape):
+    """The FP32 factors (2 x 28 floats), D^-1 (9 doubles) and two FP32 vectors (4 floats) a
+    slot of the 8 x 4-line tiles, and not the FP64 blocks (54 doubles) once more."""
+    nx, ny, nz = shape
+    g, r = _factored(shape)
+    slots = 32 * -(-ny // 8) * -(-nz // 4) * (nx + 10)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    g.precision = "mixed"
+    g.factor()
+    g.precond_apply(r)
+    torch.cuda.synchronize()
+    held = before - torch.cuda.mem_get_info()[0]
+    assert held <= slots * (4 * 56 + 8 * 9 + 2 * 4 * 4) + (12 << 20)
+    g.close()
