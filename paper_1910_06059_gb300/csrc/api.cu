@@ -948,11 +948,11 @@ bo_status bo_set_precision(bo_sim* s, int precision) {
         const bool mixed = precision == BO_PRECISION_MIXED;
         if (mixed == s->mixed) return;
         sync(s);
-        if (mixed && s->d_P32 == nullptr) {
-            dalloc(&s->d_P32, factors32_floats(s));
-            dalloc(&s->d_D32, dinv32_doubles(s));
-            dalloc(&s->d_r32, vec32_floats(s));
-            dalloc(&s->d_y32, vec32_floats(s));
+        if (mixed) {   // each on its own: an earlier call may have got only some of them
+            if (!s->d_P32) dalloc(&s->d_P32, factors32_floats(s));
+            if (!s->d_D32) dalloc(&s->d_D32, dinv32_doubles(s));
+            if (!s->d_r32) dalloc(&s->d_r32, vec32_floats(s));
+            if (!s->d_y32) dalloc(&s->d_y32, vec32_floats(s));
         }
         s->mixed = mixed;
         if (mixed) convert_factors32(s, s->stream);   // factors of an earlier bo_factor stay usable

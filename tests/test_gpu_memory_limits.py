@@ -80,3 +80,20 @@ def test_mixed_precision_holds_its_factors_once(shape):
     held = before - torch.cuda.mem_get_info()[0]
     assert held <= slots * (4 * 56 + 8 * 9 + 2 * 4 * 4) + (12 << 20)
     g.close()
+
+
+def test_mixed_precision_after_a_failed_switch():
+    """The FP32 factors (64 MB) fit, the rest (30 MB) does not; a later switch gets it."""
+    from paper_1910_06059_gb300 import _lib
+    g, r = _factored((60, 64, 64))
+    z = g.precond_apply(r)
+    with _room(80), pytest.raises(_lib.BoError, match="OOM"):
+        g.precision = "mixed"
+    assert g.precision == "fp64" and np.array_equal(g.precond_apply(r), z)
+    g.precision = "mixed"
+    got = g.precond_apply(r)
+    h, _ = _factored((60, 64, 64))
+    h.precision = "mixed"
+    assert np.array_equal(got, h.precond_apply(r))
+    g.close()
+    h.close()
