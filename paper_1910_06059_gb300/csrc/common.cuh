@@ -131,13 +131,14 @@ struct LearnSystem {
 };
 
 // FP64 sweeps (sweep64.cu): a tile of TSJ x TSK x-lines in one sweep direction
-// (lines counted in that direction), the tiles that read its results (-1:
-// none) and whether it reads the tiles before it; the plan of both directions
-// (0 forward, 1 backward) for the current block-Jacobi boxes.
+// (lines counted in that direction), the tiles that read its results (-1: none),
+// whether it reads the tile before it in j, and for each of its lines in k whether
+// it reads the line before it (bit kk of takeK; bit 0: the tile before it); the plan
+// of both directions (0 forward, 1 backward) for the current block-Jacobi boxes.
 constexpr int TSJ = 4, TSK = 3;
 struct SweepTile {
     int j0, k0, nextJ, nextK;
-    short nj, nk, depJ, depK;
+    short nj, nk, depJ, takeK;
 };
 struct SweepPlan {
     int T = 0, NL = 0;

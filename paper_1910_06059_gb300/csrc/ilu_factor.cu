@@ -76,7 +76,7 @@ k_factor_wave(SweepArgs a, const double* __restrict__ A, const unsigned* __restr
                 const int v = lane + 32 * u;
                 const bool jf = v < 9 * TSK;
                 line[u] = jf ? v / 9 : (v - 9 * TSK) / 9;
-                has[u] = v < BFACES && (jf ? t.depJ && line[u] < t.nk : t.depK && line[u] < t.nj);
+                has[u] = v < BFACES && (jf ? t.depJ && line[u] < t.nk : (t.takeK & 1) && line[u] < t.nj);
             }
             double* in = a.inbox + (size_t)rank * NL * FACE9_W + lane;
             const double sent = __longlong_as_double((long long)SENTINEL_BITS);
@@ -113,16 +113,17 @@ k_factor_wave(SweepArgs a, const double* __restrict__ A, const unsigned* __restr
             const int ln = kk * TSJ + jj;
             const bool valid = work && jj < t.nj && kk < t.nk;
             // couplings that leave the box are left out
-            const bool keep[6] = {true, jj > 0 || t.depJ, kk > 0 || t.depK,
-                                  true, jj + 1 < t.nj || t.nextJ >= 0, kk + 1 < t.nk || t.nextK >= 0};
+            const bool takeK = t.takeK >> kk & 1;
+            const bool keep[6] = {true, jj > 0 || t.depJ, takeK, true, jj + 1 < t.nj || t.nextJ >= 0,
+                                  kk + 1 < t.nk ? (t.takeK >> (kk + 1) & 1) != 0 : t.nextK >= 0};
             constexpr int from[6] = {NB_MX, NB_MY, NB_MZ, NB_PX, NB_PY, NB_PZ};
             // the neighbours' blocks: source, ring mask and place size
             const int sx = PLANE + ln * BLOCKS_W;
             const int sy = jj > 0 ? PLANE + (ln - 1) * BLOCKS_W + 9 : t.depJ ? HALO + 9 * kk : ZERO;
             const int my = jj > 0 ? 1 : t.depJ ? RING - 1 : 0, wy = jj > 0 ? BPLANE : FACE9_W;
-            const int sz = kk > 0 ? PLANE + (ln - TSJ) * BLOCKS_W + 18
-                                  : t.depK ? HALO + 9 * TSK + 9 * jj : ZERO;
-            const int mz = kk > 0 ? 1 : t.depK ? RING - 1 : 0, wz = kk > 0 ? BPLANE : FACE9_W;
+            const int sz = !takeK ? ZERO : kk > 0 ? PLANE + (ln - TSJ) * BLOCKS_W + 18
+                                                  : HALO + 9 * TSK + 9 * jj;
+            const int mz = !takeK ? 0 : kk > 0 ? 1 : RING - 1, wz = kk > 0 ? BPLANE : FACE9_W;
             const int l0 = jj + kk, j = t.j0 + jj, k = t.k0 + kk;
             const long long cbase = (long long)nx * (j + (long long)a.g.ny * k) - l0;   // cell: + l
             const double* Ae = A + (size_t)e * n;
@@ -231,7 +232,7 @@ k_scaled_blocks(SweepArgs a, const double* __restrict__ A, const double* __restr
     const int js = t.j0 + jj, ks = t.k0 + kk;
     const int j = DIR ? a.g.ny - 1 - js : js, k = DIR ? a.g.nz - 1 - ks : ks;
     const int cut = d == 1 ? cy : cz;
-    const bool keep = d == 0 || ((d == 1 ? jj > 0 || t.depJ : kk > 0 || t.depK) &&
+    const bool keep = d == 0 || ((d == 1 ? jj > 0 || t.depJ : t.takeK >> kk & 1) &&
                                  (cut == 0 || ((d == 1 ? j : k) + DIR) % cut != 0));
     const int blk = 1 + 2 * d + DIR;   // NB_MX, NB_PX, NB_MY, ... in turn
     static_assert(NB_MX == 1 && NB_PX == 2 && NB_MY == 3 && NB_PY == 4 && NB_MZ == 5 && NB_PZ == 6,
