@@ -970,22 +970,25 @@ bo_status bo_set_subdomains(bo_sim* s, int ysub, int zsub) {
         need(zsub == 0 || (zsub > 0 && zsub % 4 == 0), BO_ERR_INVALID_ARG,
              "bo_set_subdomains: zsub must be 0 or a positive multiple of 4");
         need(s->props_set, BO_ERR_STATE, "bo_set_subdomains: call bo_set_properties first");
-        if (ysub == s->ysub && zsub == s->zsub) return;
+        if (ysub == s->ysub && zsub == s->zsub && s->sweep.T > 0) return;
         sync(s);
+        auto apply = [&](int y, int z) {
+            destroy_graphs(s);     // they hold the plan's buffers
+            s->factored = false;   // the factors of the other partition are stale
+            s->ysub = y;
+            s->zsub = z;
+            setup_sweeps64(s);
+            reset_sweep_faces(s);
+            build_graphs(s);
+            sync(s);
+        };
         const int ysub0 = s->ysub, zsub0 = s->zsub;
-        s->ysub = ysub;
-        s->zsub = zsub;
         try {
-            setup_sweeps64(s);   // on failure the old plan stays
+            apply(ysub, zsub);
         } catch (...) {
-            s->ysub = ysub0;
-            s->zsub = zsub0;
+            apply(ysub0, zsub0);   // this plan fitted
             throw;
         }
-        s->factored = false;   // the factors of the other partition are stale
-        reset_sweep_faces(s);
-        build_graphs(s);
-        sync(s);
     });
 }
 

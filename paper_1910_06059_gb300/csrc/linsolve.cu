@@ -799,6 +799,7 @@ static cudaGraphExec_t capture_factor(bo_sim* s) {
 
 void build_graphs(bo_sim* s) {
     destroy_graphs(s);
+    if (s->sweep.T == 0) fail(BO_ERR_STATE, "no sweep plan: a change of the boxes ran out of memory");
     s->g_factor = capture_factor(s);
     // the FP32 sweeps' cooperative launches and the collection of residuals stay
     // with the replayed graph

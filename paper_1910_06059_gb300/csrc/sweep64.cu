@@ -405,9 +405,11 @@ void reset_tickets(bo_sim* s) {
 }
 
 // Plan of both sweeps for the current block-Jacobi boxes, filled on the
-// simulator's stream.  The new plan is complete before the old one is given up.
+// simulator's stream.  The old plan goes first, so a change of boxes needs no room for
+// two; on failure there is none (T = 0).
 void setup_sweeps64(bo_sim* s) {
     const Geom& g = s->geo;
+    free_plan(s->sweep);
     SweepPlan p;
     try {
         p.NL = g.nx + TSJ + TSK - 2;
@@ -441,7 +443,6 @@ void setup_sweeps64(bo_sim* s) {
         free_plan(p);
         throw;
     }
-    free_plan(s->sweep);
     s->sweep = p;
     s->tile_valid = false;
     // four CTAs on an SM need 144 KB of shared memory

@@ -97,3 +97,34 @@ def test_mixed_precision_after_a_failed_switch():
     assert np.array_equal(got, h.precond_apply(r))
     g.close()
     h.close()
+
+
+def test_boxes_change_without_room_for_two_plans():
+    """A sweep plan of this model takes 187 MB."""
+    g, r = _factored((60, 64, 64))
+    h, _ = _factored((60, 64, 64))
+    h.subdomains, h.subdomains_z = 0, 12
+    h.factor()
+    want = h.precond_apply(r)
+    h.close()
+    with _room(100):
+        g.subdomains_z = 12
+        g.factor()
+        assert np.array_equal(g.precond_apply(r), want)
+    g.close()
+
+
+def test_boxes_whose_plan_does_not_fit_leave_the_old_ones():
+    """Boxes of 8 layers (3 + 3 + 2) take 14 MB more than one box."""
+    from paper_1910_06059_gb300 import _lib
+    g, r = _factored((60, 64, 64))
+    z = g.precond_apply(r)
+    with _room(4), pytest.raises(_lib.BoError, match="OOM"):
+        g.subdomains_z = 8
+    assert g.subdomains_z == 0
+    g.factor()
+    assert np.array_equal(g.precond_apply(r), z)
+    g.subdomains_z = 8
+    g.factor()
+    assert not np.array_equal(g.precond_apply(r), z)
+    g.close()
