@@ -615,11 +615,12 @@ bo_status bo_ensemble_autotune_schedule(bo_ensemble* ens, double dt_probe, const
                                        double* seconds, int* small_schedule, int* streams);
 bo_status bo_ensemble_destroy(bo_ensemble* ens);
 
-/* Self-test of failure detection: runs the bounded device-side wait of the
- * wavefront sweeps on a face slot that nothing ever writes.  The wait runs
- * out after about one second, the kernel records it and returns, and the
- * call reports BO_ERR_DEVICE_TIMEOUT with *seconds (may be NULL) = the time
- * the wait took; the context stays usable.  Any other status is a failure
+/* Self-test of failure detection: runs the two bounded device-side waits of
+ * the FP64 sweeps and the factorisation, with shorter bounds, on a face slot
+ * that nothing ever writes and on a level counter that nothing advances.
+ * They run out after about a second in all, the kernel records each and
+ * returns, and the call reports BO_ERR_DEVICE_TIMEOUT with *seconds (may be
+ * NULL) = the time they took; the context stays usable.  Any other status is a failure
  * of the mechanism.  (The paper has no counterpart; Section 2.3's
  * time-step cutting is the host-side part of failure handling.) */
 bo_status bo_selftest_bounded_wait(bo_sim* sim, double* seconds);

@@ -81,8 +81,7 @@ k_factor_wave(SweepArgs a, const double* __restrict__ A, const unsigned* __restr
             double* in = a.inbox + (size_t)rank * NL * FACE9_W + lane;
             const double sent = __longlong_as_double((long long)SENTINEL_BITS);
             bool abort = false;
-            int q = 0;
-            while (warp > TSJ && ld_level(&s_begun) == 0 && ++q < WAIT_LIMIT) __nanosleep(32);
+            if (warp > TSJ) await_level<32>(&s_begun, 1, lane, a.err);
             for (int l = warp - TSJ; l < NL; l += FACE_WARPS) {
                 await_place(&s_done, l, lane, a.err);
                 bool need[2];

@@ -5,7 +5,7 @@
 #include <cmath>
 #include <vector>
 
-#include "tiles.cuh"
+#include "wavefront.cuh"
 
 namespace bo {
 
@@ -35,21 +35,40 @@ k_tile_factors(TileArgs a, SweepFactors f, double* __restrict__ P) {
     }
 }
 
-// Self-test of the bounded wait: poll a face slot that nothing writes.
-__global__ void k_wait_selftest(double* slot, int* err, long long* ns_out) {
+// Self-test of the sweeps' bounded waits with shorter bounds: a face slot that nothing
+// writes, then a level counter that nothing advances, in both its forms.  out: the time,
+// and 1 (the slot's wait set the flag and gave zeros) + 2 + 4 (the counter's waits set it).
+__global__ void k_wait_selftest(double* slot, int* err, long long* out) {
+    __shared__ int counter;
     unsigned long long t0, t1;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-    unsigned ns = 64;
-    for (long long q = 0; is_sentinel(ld_relaxed(slot)); ++q) {
-        if (q >= POLL_LIMIT) {
-            atomicExch(err, 1);
-            break;
-        }
-        __nanosleep(ns);
-        ns = ns < 1024u ? 2u * ns : 1024u;
+    const int lane = threadIdx.x;
+    if (lane == 0) counter = 0;
+    __syncwarp();
+    double* const at[1] = {slot + lane};
+    const bool need[1] = {true};
+    double v[1];
+    bool abort = false;
+    poll_faces(at, need, v, abort, lane, err, FACE_LIMIT / 4);
+    const bool polled = __all_sync(FULL, abort && v[0] == 0.0 && (lane > 0 || ld_relaxed_i(err) == 1));
+    int seen = polled ? 1 : 0;
+    if (lane == 0) atomicExch(err, 0);
+    __syncwarp();
+    await_level<32>(&counter, 1, lane, err, WAIT_LIMIT / 16);
+    __syncwarp();
+    if (lane == 0) {
+        if (ld_relaxed_i(err) == 1) seen += 2;
+        atomicExch(err, 0);
     }
+    __syncwarp();
+    await_data(&counter, 0, lane, err, WAIT_LIMIT / 16);
+    __syncwarp();
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-    *ns_out = (long long)(t1 - t0);
+    if (lane == 0) {
+        if (ld_relaxed_i(err) == 1) seen += 4;
+        out[0] = (long long)(t1 - t0);
+        out[1] = seen;
+    }
 }
 __global__ void k_fill_sentinel(double* __restrict__ p, size_t count) {
     const double sent = __longlong_as_double((long long)SENTINEL_BITS);
@@ -152,29 +171,27 @@ void read_flags_async(bo_sim* s) {
                                 cudaMemcpyDeviceToHost, s->stream));
 }
 
-// Runs one bounded face wait that can only time out; returns the wait time.
+// Runs waits that can only time out; returns the time they took.
 double wait_selftest(bo_sim* s) {
     int* err = s->d_sweep_sync + 3;   // a flag of its own: the sweeps' flag stays clear
-    long long* ns = nullptr;
+    long long* out = nullptr;
     double* slot = nullptr;           // a face slot of its own that nothing writes
     BO_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s->stream));
-    BO_CUDA(cudaMalloc(&ns, sizeof(long long)));
-    BO_CUDA(cudaMalloc(&slot, 3 * sizeof(double)));
-    k_fill_sentinel<<<1, 32, 0, s->stream>>>(slot, 3);
+    BO_CUDA(cudaMalloc(&out, 2 * sizeof(long long)));
+    BO_CUDA(cudaMalloc(&slot, 32 * sizeof(double)));
+    k_fill_sentinel<<<1, 32, 0, s->stream>>>(slot, 32);
     count_launch(s, s->stream);
-    k_wait_selftest<<<1, 1, 0, s->stream>>>(slot, err, ns);
+    k_wait_selftest<<<1, 32, 0, s->stream>>>(slot, err, out);
     count_launch(s, s->stream);
     BO_LAUNCH_CHECK("k_wait_selftest");
-    long long h = 0;
-    int e = 0;
-    BO_CUDA(cudaMemcpyAsync(&h, ns, sizeof(long long), cudaMemcpyDeviceToHost, s->stream));
-    BO_CUDA(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    long long h[2] = {0, 0};
+    BO_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
     BO_CUDA(cudaStreamSynchronize(s->stream));
-    cudaFree(ns);
+    cudaFree(out);
     cudaFree(slot);
     BO_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s->stream));
-    if (e == 0) fail(BO_ERR_STATE, "bounded-wait self-test: the wait did not run out");
-    return h * 1e-9;
+    if (h[1] != 7) fail(BO_ERR_STATE, "bounded-wait self-test: a wait did not run out as it should");
+    return h[0] * 1e-9;
 }
 
 }  // namespace bo

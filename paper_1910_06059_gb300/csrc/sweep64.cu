@@ -136,9 +136,7 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
                     if (told != l && lane == 0) st_level_release(&s_copied, l);
                     told = l;
                     if (l == NL) break;
-                    int q = 0;
-                    while ((known = begun()) + RING <= l && ++q < WAIT_LIMIT) __nanosleep(20);
-                    if (q >= WAIT_LIMIT && lane == 0) atomicExch(a.err, 1);
+                    known = __shfl_sync(FULL, await_level<20>(&s_done, l - RING + 1, lane, a.err), 0);
                 }
                 const unsigned dst = sa(ring[l & (RING - 1)]) + 16 * lane;
                 const char* f = Sp + (size_t)l * (TSJ * 96 * 8);
@@ -156,9 +154,8 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
             const int to = HALO + comp * LINES + (jf ? line : TSK + line);
             const double sent = __longlong_as_double((long long)SENTINEL_BITS);
             bool abort = false;
-            int q = 0;
             // the later levels are polled once the first has come
-            while (warp > TSJ && ld_level(&s_begun) == 0 && ++q < WAIT_LIMIT) __nanosleep(32);
+            if (warp > TSJ) await_level<32>(&s_begun, 1, lane, a.err);
             for (int l = warp - TSJ; l < NL; l += FACE_WARPS) {
                 await_place(&s_done, l, lane, a.err);
                 const int i = l - line;
@@ -169,9 +166,7 @@ k_sweep(SweepArgs a, const double* __restrict__ S, const double* __restrict__ Q,
                 if (lane < FACE_LANES) ex[to + ((l + 1) & (RING - 1)) * SLOT] = v[0];
                 if (l == 0 && lane == 0) st_level(&s_begun, 1);
                 // the next level's entries (the first one's too) are in
-                const int last = min(l + 1, NL - 1);
-                for (q = 0; ld_level_acquire(&s_copied) <= last && ++q < WAIT_LIMIT;) {}
-                if (q >= WAIT_LIMIT && lane == 0) atomicExch(a.err, 1);
+                await_data(&s_copied, min(l + 1, NL - 1), lane, a.err);
                 __syncwarp();
                 level_arrive(l & (RING - 1));
                 if (need[0]) st_relaxed(at[0], sent);

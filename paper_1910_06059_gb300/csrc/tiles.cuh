@@ -8,11 +8,7 @@ namespace bo {
 
 constexpr int TJ = 8, TK = 4;          // tile of x-lines per warp (lane = jj + TJ kk)
 constexpr unsigned long long SENTINEL_BITS = 0x7FF4DEADBEEF0001ull;  // a NaN no arithmetic yields
-// bounded waits: with the back-off below, 2^20 polls take about one second
-constexpr long long POLL_LIMIT = 1LL << 20;
-#ifndef BO_POLL_SLEEP_NS
-#define BO_POLL_SLEEP_NS 32
-#endif
+constexpr long long POLL_LIMIT = 1LL << 20;   // unit of the FP32 sweeps' bounded waits
 constexpr unsigned FULL = 0xffffffffu;
 
 // ILU(0) data in tile order: slot s = t NL + l (tile t, level l) holds NPE

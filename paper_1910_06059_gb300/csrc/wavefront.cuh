@@ -10,6 +10,7 @@ constexpr int LINES = TSJ * TSK;          // x-lines of a tile
 constexpr int RING = 8;                   // levels of the shared-memory rings (power of two)
 constexpr int FACE_WARPS = 4;             // warps that open the levels, each every fourth
 constexpr int WAIT_LIMIT = 1 << 26;       // polls of a level counter (several seconds)
+constexpr int FACE_LIMIT = 1 << 22;       // polls of a face slot, a trip to L2 each (several seconds)
 constexpr int OPEN = 32 * (TSJ + 1);      // threads that open a level
 static_assert(TSJ == 4 && TSK == 3, "one warp per j-line of the tile, three lines a warp");
 
@@ -54,12 +55,27 @@ __device__ __forceinline__ void level_arrive(int place) {
 __device__ __forceinline__ unsigned draw_tile(const SweepArgs& a) {
     return (unsigned)(atomicAdd(a.ticket, 1ull) % (unsigned long long)(a.T + gridDim.x));
 }
+// A warp's wait until a level counter has come to `least`, SLEEP ns between the polls.
+// Gives up after the bound.  Returns the counter.
+template <int SLEEP>
+__device__ __forceinline__ int await_level(const int* counter, int least, int lane, int* err,
+                                           int limit = WAIT_LIMIT) {
+    int v, q = 0;
+    while ((v = ld_level(counter)) < least && ++q < limit) __nanosleep(SLEEP);
+    if (q >= limit && lane == 0) atomicExch(err, 1);
+    return v;
+}
+// The same without a pause for a counter that announces data, until it is past `last`.
+__device__ __forceinline__ void await_data(const int* counter, int last, int lane, int* err,
+                                           int limit = WAIT_LIMIT) {
+    int q = 0;
+    while (ld_level_acquire(counter) <= last && ++q < limit) {}
+    if (q >= limit && lane == 0) atomicExch(err, 1);
+}
 // A face warp's wait before it writes the ring place of level l, read last at
 // level l - RING (done: levels begun by the compute warps).
 __device__ __forceinline__ void await_place(const int* done, int l, int lane, int* err) {
-    int q = 0;
-    while (ld_level(done) + RING <= l && ++q < WAIT_LIMIT) __nanosleep(32);
-    if (q >= WAIT_LIMIT && lane == 0) atomicExch(err, 1);
+    await_level<32>(done, l - RING + 1, lane, err);
 }
 
 // One of a face warp's values of a level: *at once it is written (need), else 0.
@@ -67,7 +83,8 @@ __device__ __forceinline__ void await_place(const int* done, int l, int lane, in
 // when another wait of the launch has given up.
 template <int N>
 __device__ __forceinline__ void poll_faces(double* const (&at)[N], const bool (&need)[N],
-                                           double (&v)[N], bool& abort, int lane, int* err) {
+                                           double (&v)[N], bool& abort, int lane, int* err,
+                                           int limit = FACE_LIMIT) {
     bool all = true;
 #pragma unroll
     for (int u = 0; u < N; ++u) {
@@ -82,7 +99,7 @@ __device__ __forceinline__ void poll_faces(double* const (&at)[N], const bool (&
             all = all && !is_sentinel(v[u]);
         }
         if ((q & 1023) == 0) {
-            const bool late = q >= 4 * POLL_LIMIT;
+            const bool late = q >= limit;
             if (late && lane == 0) atomicExch(err, 1);
             abort = __any_sync(FULL, late || ld_relaxed_i(err) != 0);
         }
