@@ -245,10 +245,10 @@ bo_status bo_get_wells(const bo_sim* sim, double* Rw, double* Dw, double* B, dou
  * its inflow at that state and BHP), which must follow this call.
  * BO_ERR_STATE before bo_set_properties; BO_ERR_INVALID_ARG for another
  * model. */
-/* Residency of the FP64 triangular sweeps' persistent CTAs: k = 1 or 2 per
- * SM (default 2).  With two, the row warps of the two CTAs on an SM share the
- * sub-partitions' FP64 pipes; with one, fewer tiles of the wavefront are in
- * flight at once.  Re-records the solver graphs.  BO_ERR_INVALID_ARG for
+/* CTAs of the FP64 triangular sweeps and the factorisation: k = 1 or 2 per SM
+ * (default 2); each takes tiles of the wavefront until none is left.  With two,
+ * the tiles on an SM share its FP64 pipes; with one, fewer tiles are in flight
+ * at once.  Re-records the solver graphs.  BO_ERR_INVALID_ARG for
  * another k, BO_ERR_STATE before bo_set_properties. */
 bo_status bo_set_sweep_ctas_per_sm(bo_sim* sim, int k);
 
@@ -441,10 +441,12 @@ bo_status bo_get_precision(const bo_sim* sim, int* precision);
  * side by side, so a sweep takes about nx + min(ny, ysub) + min(nz, zsub)
  * levels instead of nx + ny + nz.  0 means no cut in that direction, so
  * (0, 0) restores plain ILU(0).  ysub must be 0 or a positive multiple of 8
- * and zsub 0 or a positive multiple of 4 (the tile extents of the sweeps);
- * BO_ERR_INVALID_ARG otherwise.  Requires bo_set_properties; the factors of
- * an earlier bo_factor are dropped (factor again).  bo_get_subdomains
- * writes either value to a non-NULL pointer. */
+ * and zsub 0 or a positive multiple of 4 (the tile extents of the FP32
+ * sweeps); BO_ERR_INVALID_ARG otherwise.  Requires bo_set_properties; the
+ * factors of an earlier bo_factor are dropped (factor again), also when the
+ * call fails with BO_ERR_OOM (no room for the new boxes' sweep data: the old
+ * boxes are set up again).  bo_get_subdomains writes either value to a
+ * non-NULL pointer. */
 bo_status bo_set_subdomains(bo_sim* sim, int ysub, int zsub);
 bo_status bo_get_subdomains(const bo_sim* sim, int* ysub, int* zsub);
 /* Learned correction of the preconditioner, an extension of the ILU(0)-

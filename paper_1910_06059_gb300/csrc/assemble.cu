@@ -8,13 +8,13 @@
 // Kernels and their data:
 //   k_props  one thread per cell: cell quantities with derivatives (D3 duals),
 //            accumulation residual and the accumulation part of the diagonal
-//            block; writes the 28 face quantities per cell (SoA) for k_flux.
-//   k_flux   one thread per cell: the six faces of the cell in the order
-//            -z, -y, -x, +x, +y, +z; every face is evaluated in its canonical
-//            orientation (lower cell index first), so both cells see bitwise
-//            the same flux and derivatives (skew symmetry holds exactly).
-//            Each thread owns its row: residual, diagonal block and its six
-//            off-diagonal blocks; no atomics.
+//            block; writes the 28 face quantities per cell (SoA) for k_faces.
+//   k_faces  one thread per face: evaluated once, in its canonical orientation
+//            (lower cell index first), so both cells get bitwise the same flux
+//            and derivatives (skew symmetry holds exactly); writes the two
+//            off-diagonal blocks.
+//   k_flux_sums  one thread per cell: adds the cell's six faces to its residual
+//            and diagonal block in the order -z, -y, -x, +x, +y, +z; no atomics.
 //   k_wells  one block per well: connection inflow and its derivatives,
 //            well-equation residual and Schur pieces B_w, C_w, D_w.
 #include <cmath>

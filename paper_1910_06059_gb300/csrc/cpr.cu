@@ -25,13 +25,14 @@
 // GPU layout: level 0 is the 7-point pressure matrix in the Jacobian's
 // layout ap[b][n] (b: diag, -x, +x, -y, +y, -z, +z; zero where no
 // neighbour); coarser levels are CSR (what the Galerkin sums and the
-// coarsest inverse read) with an ELL copy for the V-cycle (one thread per
-// row, coalesced).  Restriction forms each level's residual once and sums
+// coarsest inverse read).  The V-cycle reads a level of short rows in an ELL copy,
+// one thread per row, and a level of long rows in CSR, eight lanes per row.
+// Restriction forms each level's residual once and sums
 // each aggregate's members in ascending order (no atomics); prolongation
 // adds each node's aggregate value.  The coarsest matrix is inverted per Newton
-// system by one CTA (Gauss-Jordan, partial pivoting) and applied as a dense
-// product.  All kernels are memory-bound streaming kernels; the V-cycle is
-// captured in the BiCGStab iteration's CUDA graph.
+// system by a cluster of 16 CTAs (Gauss-Jordan, partial pivoting; one CTA above
+// 512 unknowns) and applied as a dense product.  The V-cycle is captured in the
+// BiCGStab iteration's CUDA graph.
 #include <algorithm>
 #include <cmath>
 #include <vector>

@@ -8,8 +8,8 @@
 // of ILU(0), reached through two edges, is the cell itself or a cell outside
 // the pattern: only the diagonal blocks change,
 //     D_c = A_cc - sum_{k lower} A_ck D_k^-1 A_kc,
-// and M = (L_A + D) D^-1 (D + U_A).  The factorisation stores, in wavefront
-// order, D_c^-1 and the scaled blocks D_c^-1 A_ck (lower) and D_c^-1 A_cj
+// and M = (L_A + D) D^-1 (D + U_A).  The factorisation stores D_c^-1 and, in
+// the sweeps' orders, the scaled blocks D_c^-1 A_ck (lower) and D_c^-1 A_cj
 // (upper), so that
 //     forward  y_c = D_c^-1 r_c - sum_lower (D_c^-1 A_ck) y_k
 //     backward z_c = y_c       - sum_upper (D_c^-1 A_cj) z_j
@@ -20,8 +20,9 @@
 // iterations run in a device-side loop of a CUDA graph until the recurrence stops.
 // Every kernel reads the recurrence state and returns at once when the solve has
 // finished, so a fixed graph of several iterations can also be replayed until the
-// host sees the finished flag (timed runs, FP32 sweeps, the learned stage).  Reductions are deterministic:
-// per-block partials in a fixed grid, summed in a fixed order.
+// host sees the finished flag (timed runs, FP32 sweeps, the learned stage).
+// Reductions are deterministic: per-block partials in a fixed grid, summed in a
+// fixed order.
 #include <algorithm>
 #include <cmath>
 

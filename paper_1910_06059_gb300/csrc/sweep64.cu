@@ -20,8 +20,8 @@
 //     warp), so a level is 3 dependent products and 2 additions, 5 x 77 cycles
 //     with four warps; three chains in one lane would be 11 operations.
 //   * A CTA has four such warps (one per sub-partition) and a tile of 4 x 3
-//     x-lines (TSJ x TSK); at tile level l, line (jj, kk) handles cell i = l - jj
-//     - kk.  Results pass through a small plane in shared memory, one barrier a
+//     x-lines (TSJ x TSK), of one box or of several boxes side by side; at tile level
+//     l, line (jj, kk) handles cell i = l - jj - kk.  Results pass through a small plane in shared memory, one barrier a
 //     level; a level of a tile on its own takes 600 cycles, 304 ns.
 //   * The factors are stored lane by lane, a level's 3 KB in one piece: a copy
 //     warp brings them and the right-hand side into a ring in shared memory with
@@ -440,7 +440,7 @@ void setup_sweeps64(bo_sim* s) {
     }
     s->sweep = p;
     s->tile_valid = false;
-    // four CTAs on an SM need 144 KB of shared memory
+    // two CTAs on an SM hold about 60 KB of shared memory (a ring of 27 KB each)
     for (const void* k : {(const void*)k_sweep<true>, (const void*)k_sweep<false>})
         BO_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared));

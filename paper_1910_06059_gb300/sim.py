@@ -177,7 +177,7 @@ class Sim:
         return {q: k for k, q in L.WELL_MODEL.items()}[v.value]
 
     def set_sweep_ctas_per_sm(self, k):
-        """Persistent CTAs of the FP64 sweeps per SM (1 or 2)."""
+        """CTAs of the FP64 sweeps and the factorisation per SM (1 or 2)."""
         call("bo_set_sweep_ctas_per_sm", self.h, int(k))
 
     def set_well_model(self, name, storage=True):
