@@ -373,7 +373,8 @@ bo_status bo_get_preconditioner(const bo_sim* sim, int* kind);
 /* Schedule of the linear solve (Section 2.3.1's ILU0-BiCGStab; the paper runs
  * it as a sequence of parallel kernels, which is BO_SCHEDULE_TILED here).
  * BO_SCHEDULE_TILED (default): the wavefront-tiled sweeps and vector kernels
- * over the whole GPU, replayed as CUDA graphs of a few iterations each.
+ * over the whole GPU, as CUDA graphs: the iterations loop on the device, or a
+ * graph of a few is replayed (timing, FP32 sweeps, the learned stage).
  * BO_SCHEDULE_BLOCK: the whole solve (reduced right-hand side aside) is ONE
  * launch of ONE 256-thread CTA: triangular sweeps by levels i + j + k inside
  * the CTA, the operator, the dot products, the recurrence and its true
@@ -384,7 +385,8 @@ bo_status bo_get_preconditioner(const bo_sim* sim, int* kind);
  * FP64 ILU(0) without block-Jacobi cuts, the wells are the reduced standard
  * wells (at most 128), no learned stage runs and ceil(ny/8) ceil(nz/4) <= 128;
  * otherwise the tiled schedule runs.  bo_precond_apply follows the schedule.
- * Errors: BO_ERR_INVALID_ARG for an unknown kind or a NULL sim. */
+ * The factors are gathered for it at its launch, into a buffer of about 0.5 KB
+ * a cell that its first use allocates (BO_ERR_OOM there).  Errors: BO_ERR_INVALID_ARG for an unknown kind or a NULL sim. */
 #define BO_SCHEDULE_TILED 0
 #define BO_SCHEDULE_BLOCK 1
 bo_status bo_set_solve_schedule(bo_sim* sim, int kind);
